@@ -37,6 +37,23 @@
 // exp(i pi (z + 2 (r - k0))) is the same for every tap (q = j - (r - k0) with j integer), and
 // q^2/z is formed in FP64 for the near taps.  Everything else runs in the evaluation type T.
 //
+// k5_interp64, the FP64 evaluation at given points.  GB300 runs FP64 at 1/64 of the FP32 rate (one FP64
+// warp instruction takes the SM 16 cycles), so the FP64 instructions are what it costs:
+//  * near taps, z >= 1: one table of polynomials (FresnelTable) for d at both ends in place of the series /
+//    continued fraction, and the higher moments of all taps from the sums of t, q t, q^2 t, X and q X
+//    with t = X conj(sqrt(2z) M_0) (the integrations by parts are linear in M_0);
+//  * near taps, z < 1: the sum over the near taps (at most 26) goes inside the integral, which 64
+//    Gauss-Legendre nodes then resolve (14 cycles at most): two nodes per lane, Horner over the taps;
+//  * far taps: one division-free reciprocal per end and the sums as polynomials in tau^2;
+//  * conversions and branch decisions in FP32 and integer arithmetic;
+//  * the scalar work (square roots, divisions, the phase at u = 1) lane-parallel: a warp takes a group
+//    of points, one per lane, then evaluates them one after another with all lanes on the taps.
+// About 65 FP64 instructions per tap and lane where the form above takes 600.  4096 points, 256 taps,
+// |z| <= 84: 1000 -> 270 us, and closer to the exact sums (relative error 3e-15 against 1e-14).
+// k5_refine keeps the first form for its FP64 step: on a converged candidate whether that step is
+// taken hangs on the last bits of P, so another evaluation changes evaluation counts and, along the
+// degenerate direction, points.
+//
 // Refinement (k5_refine), from a seed (r, z), with k0 = floor(r + 1/2) of the seed kept for the
 // whole ascent so that P is smooth along the path: up to `steps` FP32 steps, then one FP64 step, of
 //   d = H^-1 grad P / P,   H^-1 = (1/(2 pi^2)) [[48, -90], [-90, 180]].
@@ -45,9 +62,11 @@
 // variance over u in [0, 1], pi^2 (dr^2/3 + dr dz/3 + 4 dz^2/45).  The step is scaled down to
 // |dr| <= 1/4, |dz| <= 1, then halved (at most three times) until P does not decrease; when no
 // such step exists the ascent stops.
+#include <algorithm>
 #include <cmath>
 
 #include "fdas_internal.cuh"
+#include "fresnel_table.cuh"
 
 namespace fdas {
 
@@ -55,10 +74,17 @@ namespace {
 
 constexpr double PI_D = 3.14159265358979323846;
 constexpr int WARPS_PER_BLOCK = 4;
+constexpr double INV_2PI = 1.0 / (2.0 * PI_D);
+constexpr int K5_WARPS = 8;              // warps per block (k5_interp64)
+constexpr int K5_GROUP_MAX = 8;          // points per warp (k5_interp64)
 
 struct GL8 {
     double x[8];
     double w[8];
+};
+struct GL64 {                            // the positive half of the 64 symmetric nodes
+    double x[32];
+    double w[32];
 };
 
 template <typename T>
@@ -364,6 +390,297 @@ __global__ void __launch_bounds__(32 * WARPS_PER_BLOCK)
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// FP64 evaluation
+
+constexpr float FAR_C64 = 12.f;
+
+template <typename V>
+__device__ __forceinline__ V from_lane(V v, int l) {
+    return __shfl_sync(0xffffffffu, v, l);
+}
+
+struct Setup64 {
+    int64_t k0;
+    double zz, dlt;     // |z|; q = j - dlt for tap offset j (folded)
+    double inv_z, inv_z_lo;   // 1/zz as a pair (zz >= 1)
+    double ks;          // sqrt(2/zz)
+    cx<double> E1;      // E(1)
+    int neg;
+};
+
+// exp(i pi x), x reduced to [-1, 1] modulo 2 (exact) first
+__device__ __forceinline__ double mod2(double x) { return x - 2.0 * rint(0.5 * x); }
+__device__ __forceinline__ cx<double> expipi64(double x) {
+    double s, c;
+    sincospi(mod2(x), &s, &c);
+    return {c, s};
+}
+
+__device__ __forceinline__ void setup64(Setup64 &c, int64_t k0, double r, double z) {
+    c.neg = z < 0.0;
+    c.k0 = k0;
+    c.zz = fabs(z);
+    const double dlt = r - (double)k0;
+    c.dlt = c.neg ? -dlt : dlt;
+    const bool big = c.zz >= 1.0;
+    c.inv_z = big ? 1.0 / c.zz : 0.0;
+    c.inv_z_lo = fma(-c.zz, c.inv_z, 1.0) * c.inv_z;
+    c.ks = big ? sqrt(2.0 / c.zz) : 0.0;
+    c.E1 = expipi64(c.zz + 2.0 * c.dlt);
+}
+__device__ __forceinline__ Setup64 from_lane(const Setup64 &s, int l) {
+    Setup64 c;
+    c.k0 = from_lane((long long)s.k0, l);
+    c.zz = from_lane(s.zz, l);
+    c.dlt = from_lane(s.dlt, l);
+    c.inv_z = from_lane(s.inv_z, l);
+    c.inv_z_lo = from_lane(s.inv_z_lo, l);
+    c.ks = from_lane(s.ks, l);
+    c.E1.re = from_lane(s.E1.re, l);
+    c.E1.im = from_lane(s.E1.im, l);
+    c.neg = from_lane(s.neg, l);
+    return c;
+}
+
+// A float widened to FP64 with integer operations (positive or negative normal values): FP64
+// conversions run at the FP64 rate.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned b = __float_as_uint(f);
+    const unsigned hi = (b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u);
+    return __hiloint2double((int)hi, (int)(b << 29));
+}
+// any float (zeros, subnormals, infinities and NaN converted)
+__device__ __forceinline__ double widen_any(float f) {
+    const unsigned e = __float_as_uint(f) & 0x7f800000u;
+    return e == 0u || e == 0x7f800000u ? (double)f : widen(f);
+}
+
+// -sgn(s) G(|s|) from the table (shared memory, [coefficient][interval]); sf: s to FP32 accuracy.
+__device__ __forceinline__ cx<double> fresnel_d(const double2 *tab, double s, float sf) {
+    const FresnelSpot at = fresnel_spot(fabsf(sf));
+    const double u = fabs(s) - widen(at.centre);
+    const double2 *p = tab + at.idx;
+    double2 c = p[(FRESNEL_TERMS - 1) * FRESNEL_INTERVALS];
+    double re = c.x, im = c.y;
+#pragma unroll
+    for (int k = FRESNEL_TERMS - 2; k >= 0; k--) {
+        c = p[k * FRESNEL_INTERVALS];
+        re = fma(re, u, c.x);
+        im = fma(im, u, c.y);
+    }
+    // the sign by integer operations on the high words
+    const int flip = (~__double2hiint(s)) & 0x80000000;
+    return {__hiloint2double(__double2hiint(re) ^ flip, __double2loint(re)),
+            __hiloint2double(__double2hiint(im) ^ flip, __double2loint(im))};
+}
+
+// Integration-by-parts end term at u = U (0 or 1), without E(u): the sums of ibp_end with 7 (S1, S2)
+// and 8 (S0) terms, real and imaginary parts as polynomials in tau^2.  vf: v in FP32.
+template <int U>
+__device__ __forceinline__ void ibp_end64(double v, float vf, double zz, cx<double> &m0, cx<double> &m1, cx<double> &m2) {
+    // 1/v: an FP32 seed (relative error e below 2^-20), then r (1 + e + e^2) (Newton's iteration, third order)
+    double r = widen(__frcp_rn(vf));
+    const double e = fma(-v, r, 1.0);
+    r = fma(r, fma(e, e, e), r);
+    const double wi = -INV_2PI * r;
+    const double tau = zz * (wi * r);
+    const double t2 = tau * tau;
+    const double s1r = fma(t2, fma(t2, fma(t2, -135135.0, 945.0), -15.0), 1.0);
+    const double s1i = tau * fma(t2, fma(t2, 10395.0, -105.0), 3.0);
+    const double s2r = fma(t2, fma(t2, fma(t2, -945945.0, 4725.0), -45.0), 1.0);
+    const double s2i = tau * fma(t2, fma(t2, 62370.0, -420.0), 6.0);
+    const double s0r = fma(-tau, s1i, 1.0), s0i = tau * s1r;
+    const double wi2 = wi * wi, wi3 = 2.0 * wi2 * wi;
+    m0 = {-wi * s0i, wi * s0r};
+    if (U == 1) {
+        m1 = {fma(wi2, s1r, m0.re), fma(wi2, s1i, m0.im)};
+        m2 = {fma(wi3, s2i, fma(wi2, s1r, m1.re)), fma(-wi3, s2r, fma(wi2, s1i, m1.im))};
+    } else {
+        m1 = {wi2 * s1r, wi2 * s1i};
+        m2 = {wi3 * s2i, -wi3 * s2r};
+    }
+}
+
+// acc += a conj(b)
+__device__ __forceinline__ void mac_conj(cx<double> &acc, cx<double> a, cx<double> b) {
+    acc.re = fma(a.re, b.re, fma(a.im, b.im, acc.re));
+    acc.im = fma(a.im, b.re, fma(-a.re, b.im, acc.im));
+}
+// E a - b
+__device__ __forceinline__ cx<double> mul_sub(cx<double> E, cx<double> a, cx<double> b) {
+    return {fma(E.re, a.re, fma(-E.im, a.im, -b.re)), fma(E.re, a.im, fma(E.im, a.re, -b.im))};
+}
+
+// P and its gradient from the three sums: dA/dr = sum X conj(2 pi i M_1) = -2 pi i Y1,
+// dA/dz = sum X conj(i pi M_2) = -i pi Y2
+struct Value64 {
+    double P, dPdr, dPdz;
+};
+__device__ __forceinline__ Value64 value_of(cx<double> A, cx<double> Y1, cx<double> Y2) {
+    const cx<double> Ar = {2.0 * PI_D * Y1.im, -2.0 * PI_D * Y1.re};
+    const cx<double> Az = {PI_D * Y2.im, -PI_D * Y2.re};
+    return {A.re * A.re + A.im * A.im, 2.0 * (A.re * Ar.re + A.im * Ar.im), 2.0 * (A.re * Az.re + A.im * Az.im)};
+}
+
+// The value at one point in FP64 (warp-collective; every lane returns the same values).  z < 0 is
+// folded by conjugation: sum X conj(M(q, z)) = conj(sum conj(X) conj(M(-q, -z))).
+// Near taps with z >= 1: with t = X conj(sqrt(2z) M_0), the higher moments of all of them follow
+// from sum t, sum q t, sum q^2 t, sum X and sum q X (the two integrations by parts are linear in M_0).
+__device__ Value64 eval64(const float2 *__restrict__ xhat, int64_t nb, int m, const Setup64 &c,
+                                const double2 *tab, const GL64 &gl) {
+    const int lane = threadIdx.x & 31;
+    const cx<double> zero = {0.0, 0.0};
+    cx<double> A = zero, Y1 = zero, Y2 = zero;                             // far taps (and the z < 1 integral)
+    const float zf = (float)c.zz, ksf = (float)c.ks;
+    const int di = (int)rint(c.dlt);                                       // q = (j - di) - df in FP32
+    const float df = (float)(c.dlt - (double)di);
+    const bool big = c.zz >= 1.0;
+    const float dfar = FAR_C64 * fmaxf(1.f, sqrtf(zf));
+    const int half = m / 2;
+    // folded offsets j with the tap inside the window: unfolded -half .. m - half - 1
+    const int64_t lo_k = c.k0 - half < 0 ? -c.k0 : -(int64_t)half;
+    const int64_t hi_k = c.k0 + (m - half) > nb ? nb - 1 - c.k0 : (int64_t)(m - half) - 1;
+    cx<double> T0 = zero, T1 = zero, T2 = zero, SX = zero, SqX = zero;     // near taps, z >= 1
+    int jl = 1, jh = 0;                                                    // near taps, z < 1
+    if (!big) {
+        jl = di + (int)ceilf(df - dfar);
+        jh = di + (int)floorf(df + zf + dfar);
+    }
+    for (int t = lane; t < m; t += 32) {
+        const int ju = t - half;
+        if (ju < lo_k || ju > hi_k) continue;
+        const int j = c.neg ? -ju : ju;
+        if (j >= jl && j <= jh) continue;
+        const float2 xv = __ldg(xhat + c.k0 + ju);
+        const cx<double> X = {widen_any(xv.x), c.neg ? -widen_any(xv.y) : widen_any(xv.y)};
+        const double q = widen_any((float)j) - c.dlt;
+        const float qf = (float)(j - di) - df;
+        if (!big || fmaxf(-qf, qf - zf) >= dfar) {
+            cx<double> a0, a1, a2, b0, b1, b2;
+            ibp_end64<1>(c.zz - q, zf - qf, c.zz, a0, a1, a2);
+            ibp_end64<0>(-q, -qf, c.zz, b0, b1, b2);
+            mac_conj(A, X, mul_sub(c.E1, a0, b0));
+            mac_conj(Y1, X, mul_sub(c.E1, a1, b1));
+            mac_conj(Y2, X, mul_sub(c.E1, a2, b2));
+        } else {
+            const double s0 = -q * c.ks, s1 = (c.zz - q) * c.ks;
+            const cx<double> d0 = fresnel_d(tab, s0, qf * ksf);
+            const cx<double> d1 = fresnel_d(tab, s1, (zf - qf) * ksf);
+            cx<double> M = mul_sub(c.E1, d1, d0);
+            if ((__double2hiint(s0) < 0) != (__double2hiint(s1) < 0)) {    // 0 < q <= z: c1 - c0 = 1 + i
+                // q^2/z with its rounding errors carried, then modulo 2
+                const double p = q * q, pl = fma(q, q, -p);
+                const double y = p * c.inv_z;
+                const double yl = fma(p, c.inv_z, -y) + fma(p, c.inv_z_lo, pl * c.inv_z);
+                double si, co;
+                sincospi(-(mod2(y) + yl), &si, &co);
+                M.re += co - si;
+                M.im += co + si;
+            }
+            const cx<double> tt = {fma(X.re, M.re, X.im * M.im), fma(X.im, M.re, -X.re * M.im)};
+            const double q2 = q * q;
+            T0 = T0 + tt;
+            T1 = {fma(q, tt.re, T1.re), fma(q, tt.im, T1.im)};
+            T2 = {fma(q2, tt.re, T2.re), fma(q2, tt.im, T2.im)};
+            SX = SX + X;
+            SqX = {fma(q, X.re, SqX.re), fma(q, X.im, SqX.im)};
+        }
+    }
+    if (big) {
+        // M_1 = K1 + (q/z) M_0, K1 = (E1 - 1)/(2 pi i z);  M_2 = E1/(2 pi i z) - M_0/(2 pi i z) + (q/z) M_1
+        const double iz = c.inv_z, rs = 0.5 * c.ks;                        // 1/sqrt(2z) = sqrt(2/z)/2
+        const cx<double> K1 = scale(iz, over_2pi_i(c.E1 - cx<double>{1.0, 0.0})), K2 = scale(iz, over_2pi_i(c.E1));
+        T0 = scale(rs, T0);
+        T1 = scale(rs * iz, T1);
+        T2 = scale(rs * iz * iz, T2);
+        A = A + T0;
+        mac_conj(Y1, SX, K1);
+        Y1 = Y1 + T1;
+        mac_conj(Y2, SX, K2);
+        mac_conj(Y2, scale(iz, SqX), K1);
+        // - conj(1/(2 pi i z)) T0 = -(i iz / (2 pi)) T0
+        Y2 = Y2 + T2 + cx<double>{iz * INV_2PI * T0.im, -iz * INV_2PI * T0.re};
+    } else {
+        // int_0^1 u^p exp(-i pi z u^2) sum_j X_j exp(2 pi i (j - dlt) u) du: lane l holds nodes +-x[l];
+        // Horner over j from jh down to jl in exp(2 pi i u)
+        const int jlo = c.neg ? (int)max((int64_t)jl, -hi_k) : (int)max((int64_t)jl, lo_k);
+        const int jhi = c.neg ? (int)min((int64_t)jh, -lo_k) : (int)min((int64_t)jh, hi_k);
+        const double xg = gl.x[lane], wg = 0.5 * gl.w[lane];
+        const double u0 = 0.5 * (1.0 - xg), u1 = 0.5 * (1.0 + xg);
+        const cx<double> w0 = expipi64(2.0 * u0), w1 = expipi64(2.0 * u1);
+        cx<double> B0 = zero, B1 = zero;
+        for (int j = jhi; j >= jlo; j--) {
+            const float2 xv = __ldg(xhat + c.k0 + (c.neg ? -j : j));
+            const cx<double> X = {widen_any(xv.x), c.neg ? -widen_any(xv.y) : widen_any(xv.y)};
+            B0 = {fma(B0.re, w0.re, fma(-B0.im, w0.im, X.re)), fma(B0.re, w0.im, fma(B0.im, w0.re, X.im))};
+            B1 = {fma(B1.re, w1.re, fma(-B1.im, w1.im, X.re)), fma(B1.re, w1.im, fma(B1.im, w1.re, X.im))};
+        }
+        if (jlo <= jhi) {
+            const double off = 2.0 * ((double)jlo - c.dlt);
+            const cx<double> e0 = scale(wg, expipi64(u0 * (off - c.zz * u0)) * B0);
+            const cx<double> e1 = scale(wg, expipi64(u1 * (off - c.zz * u1)) * B1);
+            A = A + e0 + e1;
+            Y1 = Y1 + scale(u0, e0) + scale(u1, e1);
+            Y2 = Y2 + scale(u0 * u0, e0) + scale(u1 * u1, e1);
+        }
+    }
+    A.re = warp_sum(A.re);
+    A.im = warp_sum(A.im);
+    Y1.re = warp_sum(Y1.re);
+    Y1.im = warp_sum(Y1.im);
+    Y2.re = warp_sum(Y2.re);
+    Y2.im = warp_sum(Y2.im);
+    if (c.neg) {
+        A.im = -A.im;
+        Y1.im = -Y1.im;
+        Y2.im = -Y2.im;
+    }
+    return value_of(A, Y1, Y2);
+}
+
+// One evaluation for every lane of the warp with `on` set, at (r, z) anchored at k0.
+__device__ __forceinline__ void eval64_lanes(const float2 *__restrict__ xhat, int64_t nb, int m, bool on, int64_t k0, double r,
+                                             double z, const double2 *tab, const GL64 &gl, Value64 &v) {
+    Setup64 mine{};
+    if (on) setup64(mine, k0, r, z);
+    for (unsigned todo = __ballot_sync(0xffffffffu, on); todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        const Value64 got = eval64(xhat, nb, m, from_lane(mine, l), tab, gl);
+        if ((int)(threadIdx.x & 31) == l) v = got;
+    }
+}
+
+__device__ __forceinline__ void load_table(double2 *tab) {
+    for (int i = threadIdx.x; i < FRESNEL_TERMS * FRESNEL_INTERVALS; i += blockDim.x)
+        tab[i] = reinterpret_cast<const double2 *>(fresnel_table.c)[i];
+    __syncthreads();
+}
+
+__device__ __forceinline__ int64_t anchor_of(double r) {
+    return isfinite(r) && fabs(r) < 4.5e15 ? (int64_t)floor(r + 0.5) : 0;
+}
+
+// Interpolated power in FP64, `group` consecutive points per warp.
+__global__ void __launch_bounds__(32 * K5_WARPS, 2)
+    k5_interp64(const float2 *__restrict__ xhat, int64_t nb, int m, const fdas_cand *__restrict__ pts,
+                const int64_t *__restrict__ k0s, int n, int group, double *__restrict__ out, GL64 gl) {
+    extern __shared__ double2 tab[];
+    load_table(tab);
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * K5_WARPS + (threadIdx.x >> 5)) * group + lane;
+    const bool mine = lane < group && i < n;
+    const double r = mine ? pts[i].r : NAN, z = mine ? pts[i].z : NAN;
+    const int64_t k0 = mine && k0s ? k0s[i] : anchor_of(r);
+    Value64 v = {NAN, NAN, NAN};
+    eval64_lanes(xhat, nb, m, point_ok(r, z, k0), k0, r, z, tab, gl, v);
+    if (mine) {
+        out[3 * (size_t)i + 0] = v.P;
+        out[3 * (size_t)i + 1] = v.dPdr;
+        out[3 * (size_t)i + 2] = v.dPdz;
+    }
+}
+
 // The preconditioned step (see the header comment); false when there is none.
 __device__ __forceinline__ bool ascent_step(double P, double gr, double gz, double &dr, double &dz) {
     if (!(P > 0.0)) return false;
@@ -459,16 +776,42 @@ GL8 gl8() {
 
 unsigned blocks_for(int n) { return (unsigned)((n + WARPS_PER_BLOCK - 1) / WARPS_PER_BLOCK); }
 
+const GL64 &gl64() {
+    static const GL64 g = [] {
+        double x[64], w[64];
+        gauss_legendre(64, x, w);
+        GL64 t;
+        for (int i = 0; i < 32; i++) {
+            t.x[i] = x[i];
+            t.w[i] = w[i];
+        }
+        return t;
+    }();
+    return g;
+}
+
+// Points per warp: as many as leave about 12 warps per SM busy (a group shares the scalar FP64 work).
+int group_size(const Plan &p, int n) {
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device >= 0 ? p.device : 0);
+    return std::max(1, std::min(K5_GROUP_MAX, n / (12 * std::max(sms, 1))));
+}
+constexpr size_t TABLE_BYTES = sizeof(double2) * FRESNEL_TERMS * FRESNEL_INTERVALS;
+static_assert(TABLE_BYTES <= 48 * 1024, "the table fits the default shared-memory limit");
+
+
 }  // namespace
 
 cudaError_t launch_interp(Plan &p, const float2 *d_x, const fdas_cand *d_pts, const int64_t *d_k0, int n, bool fp64,
                           double *d_out, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    const GL8 g = gl8();
-    if (fp64)
-        k5_interp<double><<<blocks_for(n), 32 * WARPS_PER_BLOCK, 0, st>>>(d_x, p.nb, p.m, d_pts, d_k0, n, d_out, g);
-    else
-        k5_interp<float><<<blocks_for(n), 32 * WARPS_PER_BLOCK, 0, st>>>(d_x, p.nb, p.m, d_pts, d_k0, n, d_out, g);
+    if (fp64) {
+        const int g = group_size(p, n);
+        const unsigned blocks = (unsigned)((n + (int64_t)K5_WARPS * g - 1) / (K5_WARPS * g));
+        k5_interp64<<<blocks, 32 * K5_WARPS, TABLE_BYTES, st>>>(d_x, p.nb, p.m, d_pts, d_k0, n, g, d_out, gl64());
+    } else {
+        k5_interp<float><<<blocks_for(n), 32 * WARPS_PER_BLOCK, 0, st>>>(d_x, p.nb, p.m, d_pts, d_k0, n, d_out, gl8());
+    }
     p.prof.launches += 1;
     return cudaGetLastError();
 }
