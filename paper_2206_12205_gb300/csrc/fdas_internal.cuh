@@ -78,7 +78,7 @@ struct Plan {
     float2 *d_twn_hi;      // W_N^(j << TW_LO_BITS), j < max(1, N >> TW_LO_BITS)
     float2 *d_G;           // [K][S] FP32 template bank
     __nv_bfloat162 *d_Gbf; // [K][S] BF16 template bank, stage-1 operand order (tensor path)
-    void *d_tcF;           // BF16 K-major DFT operand images: split hi, split lo, F1, F2 (4 x 32 KB)
+    void *d_tcF;           // BF16 K-major DFT operand images: F1, F2 and their rounding remainders (4 x 32 KB)
     __half2 *d_Gh;         // [K][S] FP16 template bank times S, stage-1 operand order
     void *d_tcFh;          // FP16 K-major DFT operand images F1, F2 (2 x 32 KB)
     void *d_dimg;          // direct paths: conj(taps) real-ified, K-major operand image (BF16 or E4M3)
@@ -93,7 +93,6 @@ struct Plan {
     bool borrowed;         // template bank and tables belong to another plan (a batch's group leader)
     // launch parameters chosen by the batch autotuner (0: built-in heuristic)
     int tune_zb;           // FP32 path: templates per correlation CTA
-    int tune_cta_per_sm;   // split-BF16 path: persistent CTAs per SM
     std::string last_error;
     mutable Profiler prof;
 };

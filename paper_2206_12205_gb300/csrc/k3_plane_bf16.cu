@@ -572,23 +572,15 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc(const uint4 *__rest
 // v_hi + v_lo with v_hi = bf16(v), v_lo = bf16(v - v_hi) (about 16 significant bits), and each
 // product as a_hi b_hi + a_lo b_hi + a_hi b_lo (the a_lo b_lo term, ~2^-18 relative, is
 // dropped): three MMAs per K step, FP32 accumulation in TMEM.  Inputs are the FP32 segment
-// spectra and the FP32 templates; the plane is stored in FP32.  Same transposed two-stage
-// DFT as above, one item at a time per CTA (synchronous), 8 warps.
-// B1 tiles (stage-1 A operand, K-major): core matrices 144 B apart along M, 16 x 144 B along K
-constexpr uint32_t B_SBO = 144, B_LBO = 16 * B_SBO;
-constexpr uint32_t B_TILE = 16 * B_LBO;                      // 36 KB
-// A2 tiles (stage-2 A operand, K-major): 128 B along M, 2064 B (16 mod 128) along K
-constexpr uint32_t A2_SBO = 128, A2_LBO = 16 * 128 + 16;
-constexpr uint32_t A2_TILE = 16 * A2_LBO;                    // 32.25 KB
-constexpr int SP_THREADS = 256;
-constexpr uint32_t SP_OFF_FHI = 0;
-constexpr uint32_t SP_OFF_FLO = TILE_BYTES;
-constexpr uint32_t SP_OFF_AHI = 2 * TILE_BYTES;                      // A tiles (B1 layout / A2 layout)
-constexpr uint32_t SP_TILE = B_TILE > A2_TILE ? B_TILE : A2_TILE;
-constexpr uint32_t SP_OFF_ALO = SP_OFF_AHI + SP_TILE;
-constexpr uint32_t SP_OFF_BAR = SP_OFF_ALO + SP_TILE;
-constexpr uint32_t SP_SMEM = SP_OFF_BAR + 64;
-
+// spectra and the FP32 templates; the plane is stored in FP32.
+// The transposed two-stage DFT and the roles of k3_plane_tc, with
+//   producer:    x = conj(Yhat_j) G_z in FP32, split, into the A1 columns (64 hi, 64 lo)
+//   epilogue 1:  W_S^{n2 k1} D1 in FP32, split, into two A2 tiles (hi, lo)
+//   epilogue 2:  |D2|^2 -> FP32 plane
+// F1, F2 hi and lo take 128 KB of shared memory, so A1 and A2 have one slot each: stage 1 of item
+// k + 1 runs while epilogue 1 writes A2 of item k, stage 2 of item k while the producer writes A1 of
+// item k + 2.  The MMAs bound it: 48 of 64 cycles an item = 3072 cycles.  N = 2^21, 85 templates,
+// 256 taps: 0.849 ms with one item at a time and a CTA-wide barrier between the steps.
 __device__ __forceinline__ void split_bf16x2(float re, float im, uint32_t &hi, uint32_t &lo) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(re, im);
     const float2 hf = __bfloat1622float2(h);
@@ -597,155 +589,317 @@ __device__ __forceinline__ void split_bf16x2(float re, float im, uint32_t &hi, u
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
-__global__ void __launch_bounds__(SP_THREADS, 1) k3_plane_tc_split(const float2 *__restrict__ Y,
+// Registers at launch 72 a thread; 128 x 56 + 256 x 88 + 256 x 72 + 256 x 64 = 896 x 72 (the
+// producers hold the FP32 loads of the next eight points while they split the current ones).
+constexpr int SP_REG_MMA = 56, SP_REG_PROD = 88, SP_REG_E1 = 72, SP_REG_E2 = 64;
+static_assert(128 * SP_REG_MMA + 256 * (SP_REG_PROD + SP_REG_E1 + SP_REG_E2) == WS_THREADS * REG_LAUNCH,
+              "register split must add up to the launch allocation");
+constexpr uint32_t SP_OFF_A2 = 4 * TILE_BYTES;               // F1, F2 hi, then F1, F2 lo; A2 hi, lo
+constexpr uint32_t SP_OFF_TWS = 6 * TILE_BYTES;
+constexpr uint32_t SP_OFF_BAR = SP_OFF_TWS + (TC_R / 2) * TC_R * 16;
+constexpr uint32_t SP_SMEM = SP_OFF_BAR + 256;
+static_assert(SP_SMEM <= 227 * 1024, "one CTA per SM");
+
+// a1_full, a1_free: one pair per half of the A1 columns (the half a producer warp writes), so that the
+// first half of an item goes in while the MMAs still read the second half of the item before it.
+struct SpBars {
+    uint64_t a1_full[2], a1_free[2], d1_full[3], b2_full, a2_free, d2_full[3], d_free[3], drain[2];
+};
+
+__global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 *__restrict__ Y,
                                                                    const float2 *__restrict__ G,
-                                                                   const uint4 *__restrict__ Fhi_img,
-                                                                   const uint4 *__restrict__ Flo_img,
+                                                                   const uint4 *__restrict__ Fimg,
                                                                    const float2 *__restrict__ tw,
                                                                    float *__restrict__ plane, int K, int64_t nb, int L,
                                                                    int64_t n_items, int n_groups, int64_t items_per_cta,
                                                                    int32_t *__restrict__ status) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + SP_OFF_BAR);
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + SP_OFF_BAR + 16);
+    SpBars *bars = reinterpret_cast<SpBars *>(smem + SP_OFF_BAR);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + SP_OFF_BAR + sizeof(SpBars));
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + SP_OFF_BAR + sizeof(SpBars) + 8);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
     if (warp == 0) {
-        tc::tmem_alloc(tslot, TC_N);
+        tc::tmem_alloc(tslot, WS_TMEM_COLS);
         tc::tmem_relinquish();
     }
-    if (tid == 0) tc::mbar_init(bar, 1);
-    for (int i = tid; i < (int)(TILE_BYTES / 16); i += SP_THREADS) {
-        reinterpret_cast<uint4 *>(smem + SP_OFF_FHI)[i] = __ldg(Fhi_img + i);
-        reinterpret_cast<uint4 *>(smem + SP_OFF_FLO)[i] = __ldg(Flo_img + i);
+    if (tid == 0) {
+        for (int s = 0; s < 2; s++) {
+            tc::mbar_init(&bars->a1_full[s], WS_PRODUCERS / 2);
+            tc::mbar_init(&bars->a1_free[s], 1);
+        }
+        tc::mbar_init(&bars->b2_full, 256);
+        tc::mbar_init(&bars->a2_free, 1);
+        for (int s = 0; s < 3; s++) {
+            tc::mbar_init(&bars->d1_full[s], 1);
+            tc::mbar_init(&bars->d2_full[s], 1);
+            tc::mbar_init(&bars->d_free[s], 256);
+        }
+        tc::mbar_init(&bars->drain[0], 1);
+        tc::mbar_init(&bars->drain[1], 1);
+        *abort_flag = 0;
+    }
+    for (int i = tid; i < (int)(4 * TILE_BYTES / 16); i += WS_THREADS) reinterpret_cast<uint4 *>(smem)[i] = __ldg(Fimg + i);
+    for (int e = tid; e < (TC_R / 2) * TC_R; e += WS_THREADS) {
+        const int kp = e / TC_R, n2 = e % TC_R;
+        const float2 a = __ldg(tw + (2 * kp) * TC_R + n2), b = __ldg(tw + (2 * kp + 1) * TC_R + n2);
+        reinterpret_cast<float4 *>(smem + SP_OFF_TWS)[e] = make_float4(a.x, b.x, a.y, b.y);
     }
     tc::fence_proxy_async_smem();
     tc::fence_before_thread_sync();
     __syncthreads();
     tc::fence_after_thread_sync();
-    const uint32_t tD = *tslot;
-    const uint32_t idesc = tc::idesc_bf16_f32(TC_M, TC_N);
-    const uint32_t fhi = tc::smem_u32(smem + SP_OFF_FHI), flo = tc::smem_u32(smem + SP_OFF_FLO);
-    const uint32_t ahi = tc::smem_u32(smem + SP_OFF_AHI), alo = tc::smem_u32(smem + SP_OFF_ALO);
-    unsigned char *sAhi = smem + SP_OFF_AHI, *sAlo = smem + SP_OFF_ALO;
-    const int quad = warp & 3, half = warp >> 2;
-    const int lrow = 32 * quad + lane, zl_e = lrow >> 6, idx = lrow & 63;
-    const uint32_t lane_base = (uint32_t)(32 * quad) << 16;
-    uint32_t phase = 0;
-    bool ok = true;
 
-    auto mma3 = [&](uint32_t a_hi, uint32_t a_lo, uint32_t albo, uint32_t asbo) {
-#pragma unroll 1
-        for (int s = 0; s < TC_K / 16; s++) {
-            const uint64_t dh = tc::smem_desc(a_hi + s * 2 * albo, albo, asbo);
-            const uint64_t dl = tc::smem_desc(a_lo + s * 2 * albo, albo, asbo);
-            const uint64_t bh = tc::smem_desc(fhi + s * 2 * F_LBO, F_LBO, F_SBO);
-            const uint64_t bl = tc::smem_desc(flo + s * 2 * F_LBO, F_LBO, F_SBO);
-            tc::mma_bf16(tD, dh, bh, idesc, s > 0 ? 1u : 0u);
-            tc::mma_bf16(tD, dl, bh, idesc, 1u);
-            tc::mma_bf16(tD, dh, bl, idesc, 1u);
-        }
-        tc::mma_commit(bar);
-    };
-
+    const uint32_t tbase = *tslot;
     const int64_t it0 = (int64_t)blockIdx.x * items_per_cta;
     const int64_t it1 = min(n_items, it0 + items_per_cta);
-    for (int64_t it = it0; it < it1 && ok; it++) {
-        const int64_t j = it / n_groups;
-        const int z0 = (int)(it % n_groups) * TC_G;
-        // ---- x = conj(Yhat_j) G_z in FP32, split, as the stage-1 A tile (B1 layout)
-        {
-            const int n2q = tid & 15, n1q = tid >> 4;
-            const float2 *Yj = Y + j * TC_S_BF16;
+    const int64_t n_my = it1 - it0;
+    const int64_t n_seg = n_items / n_groups;           // items are pair * n_seg + segment
+    const int quad = warp & 3;                          // TMEM lane quadrant this warp may access
+    const uint32_t lane_base = (uint32_t)(32 * quad) << 16;
+
+    if (warp < WS_P0) {
+        // ---------------------------------------------------------------- MMA issuers (as in k3_plane_tc)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SP_REG_MMA));
+        if (warp < 2 && n_my > 0) {
+            auto wait = [&](uint64_t *bar, uint32_t parity) {
+                return __shfl_sync(0xffffffffu, (int)ws_wait(bar, parity, abort_flag), 0) != 0;
+            };
+            int s3 = 0, u3 = 0;
+            const uint32_t id = tc::idesc_bf16_f32(TC_M, TC_N);
+            if (warp == 0) {
+                const uint64_t fh = tc::smem_desc(tc::smem_u32(smem), F_LBO, F_SBO);
+                const uint64_t fl = tc::smem_desc(tc::smem_u32(smem + 2 * TILE_BYTES), F_LBO, F_SBO);
+                for (int64_t k = 0; k < n_my; k++) {
+                    if (u3 >= 1 && !wait(&bars->d_free[s3], (uint32_t)((u3 - 1) & 1))) break;
+                    const uint32_t d = tbase + (uint32_t)s3 * TC_N, ah = tbase + COL_A1, al = ah + TC_K / 2;
+                    bool ok = true;
 #pragma unroll
-            for (int zl = 0; zl < TC_G; zl++) {
-                const int z = z0 + zl;
-                const float2 *Gz = G + (int64_t)(z < K ? z : 0) * TC_S_BF16;
-                uint32_t wh[4][4], wl[4][4];
+                    for (int hf = 0; hf < 2; hf++) {
+                        ok = ok && wait(&bars->a1_full[hf], (uint32_t)(k & 1));
+                        if (!ok) break;
+                        tc::fence_after_thread_sync();
 #pragma unroll
-                for (int q = 0; q < 4; q++) {
-#pragma unroll
-                    for (int e = 0; e < 4; e++) {
-                        const int n = 64 * (4 * n1q + q) + 4 * n2q + e;
-                        const float2 y = __ldg(Yj + n);
-                        const float2 g = z < K ? __ldg(Gz + n) : make_float2(0.f, 0.f);
-                        split_bf16x2(y.x * g.x + y.y * g.y, y.x * g.y - y.y * g.x, wh[e][q], wl[e][q]);
+                        for (int s = hf * TC_K / 32; s < (hf + 1) * TC_K / 32; s++) {
+                            const uint64_t f = (uint64_t)(s * 2 * F_LBO / 16);
+                            tc::mma_tmem_a_warp(d, ah + 8 * s, fh + f, id, s > 0 ? 1u : 0u);
+                            tc::mma_tmem_a_warp(d, al + 8 * s, fh + f, id, 1u);
+                            tc::mma_tmem_a_warp(d, ah + 8 * s, fl + f, id, 1u);
+                        }
+                        tc::mma_commit_warp(&bars->a1_free[hf]);
+                    }
+                    if (!ok) break;
+                    tc::mma_commit_warp(&bars->d1_full[s3]);
+                    if (++s3 == 3) {
+                        s3 = 0;
+                        u3++;
                     }
                 }
+            } else {
+                const uint32_t id2 = id | (1u << 15);                          // A MN-major
+                const uint64_t fh = tc::smem_desc(tc::smem_u32(smem + TILE_BYTES), F_LBO, F_SBO);
+                const uint64_t fl = tc::smem_desc(tc::smem_u32(smem + 3 * TILE_BYTES), F_LBO, F_SBO);
+                const uint64_t ah = tc::smem_desc(tc::smem_u32(smem + SP_OFF_A2), A2_CK, A2_CM);
+                const uint64_t al = tc::smem_desc(tc::smem_u32(smem + SP_OFF_A2 + TILE_BYTES), A2_CK, A2_CM);
+                for (int64_t k = 0; k < n_my; k++) {
+                    if (!wait(&bars->b2_full, (uint32_t)(k & 1))) break;       // A2 ready, D1 read
+                    tc::fence_after_thread_sync();
+                    const uint32_t d = tbase + (uint32_t)s3 * TC_N;
 #pragma unroll
-                for (int e = 0; e < 4; e++) {
-                    const int c = zl * TC_R + 4 * n2q + e;
-                    const uint32_t off = tc::kmajor_offset_strided(B_SBO, B_LBO, c, 8 * n1q);
-                    *reinterpret_cast<uint4 *>(sAhi + off) = make_uint4(wh[e][0], wh[e][1], wh[e][2], wh[e][3]);
-                    *reinterpret_cast<uint4 *>(sAlo + off) = make_uint4(wl[e][0], wl[e][1], wl[e][2], wl[e][3]);
+                    for (int s = 0; s < TC_K / 16; s++) {
+                        const uint64_t f = (uint64_t)(s * 2 * F_LBO / 16), a = (uint64_t)(s * 2 * A2_CK / 16);
+                        tc::mma_bf16_warp(d, ah + a, fh + f, id2, s > 0 ? 1u : 0u);
+                        tc::mma_bf16_warp(d, al + a, fh + f, id2, 1u);
+                        tc::mma_bf16_warp(d, ah + a, fl + f, id2, 1u);
+                    }
+                    tc::mma_commit_warp(&bars->a2_free);
+                    tc::mma_commit_warp(&bars->d2_full[s3]);
+                    if (++s3 == 3) {
+                        s3 = 0;
+                        u3++;
+                    }
                 }
             }
+            // drain: every MMA this warp issued has completed before TMEM can be released
+            tc::mma_commit_warp(&bars->drain[warp]);
+            tc::mbar_wait_bounded(&bars->drain[warp], 0, WAIT_CYCLES);
         }
-        tc::fence_proxy_async_smem();
-        tc::fence_before_thread_sync();
-        __syncthreads();
-        tc::fence_after_thread_sync();
-        if (tid == 0) mma3(ahi, alo, B_LBO, B_SBO);
-        ok = __syncthreads_and(tc::mbar_wait_bounded(bar, phase, WAIT_CYCLES));
-        phase ^= 1;
-        if (!ok) break;
-        tc::fence_after_thread_sync();
-        // ---- twiddle, split, as the stage-2 A tile (A2 layout); row (z, k1), K (n2, s)
-#pragma unroll 1
-        for (int ch = 0; ch < 4; ch++) {
-            uint32_t rr[16];
-            tc::tmem_ld16(tD + lane_base + 64 * half + 16 * ch, rr);
-            tc::tmem_ld_wait();
+        __syncwarp();
+    } else if (warp < WS_E1) {
+        // ---------------------------------------------------------------- producer
+        // thread -> A1 row (z1, n2) (interleaved order), n1 in [32 hp, 32 hp + 32), eight at a time
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SP_REG_PROD));
+        const int hp = (warp - WS_P0) >> 2;
+        const int z1 = (lane >> 4) & 1, n2 = 16 * quad + (lane & 15);
+        int64_t j = it0 % n_seg;
+        int grp = (int)(it0 / n_seg);
+        const uint32_t a1 = tbase + lane_base + COL_A1 + 32 * hp;
+        float2 y[8], g[8];
+        auto load = [&](int64_t jj, int gg, int i) {        // the points n1 = 32 hp + 8 i + e
+            const int z = gg * TC_G + z1;
+            const float2 *Yp = Y + jj * TC_S_BF16 + (32 * hp + 8 * i) * TC_R + n2;
+            const float2 *Gp = G + (int64_t)(z < K ? z : 0) * TC_S_BF16 + (32 * hp + 8 * i) * TC_R + n2;
 #pragma unroll
-            for (int q = 0; q < 8; q++) {
-                const int k1 = 32 * half + 8 * ch + q;
-                const float2 t = __ldg(tw + idx * TC_R + k1);
-                const float re = __uint_as_float(rr[2 * q]), im = __uint_as_float(rr[2 * q + 1]);
-                uint32_t h, l;
-                split_bf16x2(re * t.x - im * t.y, re * t.y + im * t.x, h, l);
-                const uint32_t off = tc::kmajor_offset_strided(A2_SBO, A2_LBO, zl_e * TC_R + k1, 2 * idx);
-                *reinterpret_cast<uint32_t *>(sAhi + off) = h;
-                *reinterpret_cast<uint32_t *>(sAlo + off) = l;
+            for (int e = 0; e < 8; e++) {
+                y[e] = __ldg(Yp + e * TC_R);
+                g[e] = __ldg(Gp + e * TC_R);
             }
+        };
+        if (n_my > 0) load(j, grp, 0);
+        for (int64_t k = 0; k < n_my; k++) {
+            const bool live = grp * TC_G + z1 < K;
+            int64_t jn = j + 1;
+            int gn = grp;
+            if (jn == n_seg) {
+                jn = 0;
+                gn++;
+            }
+            bool ok = true;
+#pragma unroll
+            for (int i = 0; i < 4; i++) {
+                float2 x[8];
+#pragma unroll
+                for (int e = 0; e < 8; e++)
+                    x[e] = live ? make_float2(y[e].x * g[e].x + y[e].y * g[e].y, y[e].x * g[e].y - y[e].y * g[e].x)
+                                : make_float2(0.f, 0.f);
+                if (i < 3) load(j, grp, i + 1);
+                else if (k + 1 < n_my) load(jn, gn, 0);
+                if (i == 0 && k >= 1) {
+                    ok = ws_wait(&bars->a1_free[hp], (uint32_t)((k - 1) & 1), abort_flag);
+                    if (!ok) break;
+                    tc::fence_after_thread_sync();
+                }
+                // columns of chunks 2 i', 2 i' + 1 (i' = 4 hp + i): points e = 0, 2, 4, 6, then 1, 3, 5, 7
+                uint32_t hi[8], lo[8];
+#pragma unroll
+                for (int c = 0; c < 2; c++)
+#pragma unroll
+                    for (int q = 0; q < 2; q++) {
+                        const float2 u = x[c + 4 * q], v = x[c + 4 * q + 2];
+                        split_bf16x2(u.x, v.x, hi[4 * c + 2 * q], lo[4 * c + 2 * q]);
+                        split_bf16x2(u.y, v.y, hi[4 * c + 2 * q + 1], lo[4 * c + 2 * q + 1]);
+                    }
+                tc::tmem_st8(a1 + 8 * i, hi);
+                tc::tmem_st8(a1 + TC_K / 2 + 8 * i, lo);
+            }
+            if (!ok) break;
+            tc::tmem_st_wait();
+            tc::fence_before_thread_sync();
+            mbar_arrive(&bars->a1_full[hp]);
+            j = jn;
+            grp = gn;
         }
-        tc::fence_proxy_async_smem();
-        tc::fence_before_thread_sync();
-        __syncthreads();
-        tc::fence_after_thread_sync();
-        if (tid == 0) mma3(ahi, alo, A2_LBO, A2_SBO);
-        ok = __syncthreads_and(tc::mbar_wait_bounded(bar, phase, WAIT_CYCLES));
-        phase ^= 1;
-        if (!ok) break;
-        tc::fence_after_thread_sync();
-        // ---- |X|^2 -> FP32 plane; thread row (z, k1), columns (k2, p)
-        {
-            const int z = z0 + zl_e;
-            const int64_t r0 = j * L;
-#pragma unroll 1
-            for (int ch = 0; ch < 4; ch++) {
-                uint32_t rr[16];
-                tc::tmem_ld16(tD + lane_base + 64 * half + 16 * ch, rr);
+    } else if (warp < WS_E2) {
+        // ---------------------------------------------------------------- epilogue 1
+        // thread -> D1 row (z1, n2) (interleaved order), k1 in [32 h, 32 h + 32)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SP_REG_E1));
+        const int h = (warp - WS_E1) >> 2;
+        const int z1 = (lane >> 4) & 1, n2 = 16 * quad + (lane & 15);
+        const float4 *tws = reinterpret_cast<const float4 *>(smem + SP_OFF_TWS) + 16 * h * TC_R + n2;
+        const uint32_t a2_row = (uint32_t)(8 * z1 + 4 * h) * A2_CM + (uint32_t)(n2 >> 3) * A2_CK + (n2 & 7) * 16;
+        unsigned char *a2 = smem + SP_OFF_A2 + a2_row;
+        int s3 = 0, u3 = 0;
+        for (int64_t k = 0; k < n_my; k++) {
+            const uint32_t dcol = (uint32_t)s3 * TC_N;
+            if (!ws_wait(&bars->d1_full[s3], (uint32_t)(u3 & 1), abort_flag)) break;
+            if (k >= 1 && !ws_wait(&bars->a2_free, (uint32_t)((k - 1) & 1), abort_flag)) break;
+            tc::fence_after_thread_sync();
+#pragma unroll
+            for (int gg = 0; gg < 2; gg++) {
+                uint32_t rr[16], ri[16];
+                tc::tmem_ld16(tbase + lane_base + dcol + 32 * h + 16 * gg, rr);
+                tc::tmem_ld16(tbase + lane_base + dcol + TC_R + 32 * h + 16 * gg, ri);
                 tc::tmem_ld_wait();
 #pragma unroll
-                for (int q = 0; q < 8; q++) {
-                    const int k2 = 32 * half + 8 * ch + q;
-                    const int t = idx + 64 * k2;
-                    if (z < K && t < L && r0 + t < nb) {
-                        const float re = __uint_as_float(rr[2 * q]), im = __uint_as_float(rr[2 * q + 1]);
-                        plane[(int64_t)z * nb + r0 + t] = re * re + im * im;
+                for (int g2 = 0; g2 < 2; g2++) {
+                    const int g = 2 * gg + g2;
+                    uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+                    for (int i = 0; i < 4; i++) {
+                        const float4 t = tws[(4 * g + i) * TC_R];
+                        const float2 wx = make_float2(t.x, t.y), wy = make_float2(t.z, t.w);
+                        const float2 dr = u2f2(rr[8 * g2 + 2 * i], rr[8 * g2 + 2 * i + 1]);
+                        const float2 di = u2f2(ri[8 * g2 + 2 * i], ri[8 * g2 + 2 * i + 1]);
+                        const float2 q = __fmul2_rn(di, wy);
+                        const float2 yr = __ffma2_rn(dr, wx, make_float2(-q.x, -q.y));
+                        const float2 yi = __ffma2_rn(dr, wy, __fmul2_rn(di, wx));
+                        split_bf16x2(yr.x, yr.y, rh[i], rl[i]);
+                        split_bf16x2(yi.x, yi.y, ih[i], il[i]);
                     }
+                    *reinterpret_cast<uint4 *>(a2 + g * A2_CM) = make_uint4(rh[0], rh[1], rh[2], rh[3]);
+                    *reinterpret_cast<uint4 *>(a2 + g * A2_CM + 8 * A2_CK) = make_uint4(ih[0], ih[1], ih[2], ih[3]);
+                    *reinterpret_cast<uint4 *>(a2 + TILE_BYTES + g * A2_CM) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+                    *reinterpret_cast<uint4 *>(a2 + TILE_BYTES + g * A2_CM + 8 * A2_CK) = make_uint4(il[0], il[1], il[2], il[3]);
                 }
             }
+            tc::fence_before_thread_sync();
+            tc::fence_proxy_async_smem();
+            mbar_arrive(&bars->b2_full);
+            if (++s3 == 3) {
+                s3 = 0;
+                u3++;
+            }
         }
-        tc::fence_before_thread_sync();
-        __syncthreads();
-    }
-    if (!ok) {
-        if (tid == 0) atomicOr(status, FDAS_DEV_TIMEOUT);
-        tc::mbar_wait_bounded(bar, phase ^ 1, WAIT_CYCLES);   // the MMAs still in flight
+    } else {
+        // ---------------------------------------------------------------- epilogue 2
+        // thread -> D2 row (zl, k1 = idx), k2 in [32 h, 32 h + 32), 16 at a time
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(SP_REG_E2));
+        const int h = (warp - WS_E2) >> 2;
+        const int lrow = 32 * quad + lane, zl = lrow >> 6, idx = lrow & 63;
+        const int kl = L / TC_R;                        // k2 < L / 64  <=>  bin t = k1 + 64 k2 < L
+        int64_t j = it0 % n_seg;
+        int grp = (int)(it0 / n_seg);
+        int slot = 0, u3 = 0;
+        for (int64_t k = 0; k < n_my; k++) {
+            const uint32_t dcol = (uint32_t)slot * TC_N;
+            if (!ws_wait(&bars->d2_full[slot], (uint32_t)(u3 & 1), abort_flag)) break;
+            tc::fence_after_thread_sync();
+            const int z = grp * TC_G + zl;
+            const int64_t r0 = j * L;
+            if (++j == n_seg) {                         // the next item
+                j = 0;
+                grp++;
+            }
+            // stored k2: k2 < kmax, from t < L, r0 + t < nb and z < K
+            int kmax = kl;
+            if (z >= K) {
+                kmax = 0;
+            } else if (r0 + L > nb) {
+                const int64_t rest = nb - r0 - idx;
+                const int64_t kr = (rest + TC_R - 1) / TC_R;
+                kmax = rest <= 0 ? 0 : (kr < (int64_t)kl ? (int)kr : kl);
+            }
+            kmax -= 32 * h;
+            float *prow = plane + (int64_t)(z < K ? z : 0) * nb + r0 + idx + 64 * 32 * h;
+#pragma unroll
+            for (int gg = 0; gg < 2; gg++) {
+                uint32_t rr[16], ri[16];
+                tc::tmem_ld16(tbase + lane_base + dcol + 32 * h + 16 * gg, rr);
+                tc::tmem_ld16(tbase + lane_base + dcol + TC_R + 32 * h + 16 * gg, ri);
+                tc::tmem_ld_wait();
+                if (gg == 1) {
+                    tc::fence_before_thread_sync();
+                    mbar_arrive(&bars->d_free[slot]);                    // accumulator slot drained
+                }
+#pragma unroll
+                for (int i = 0; i < 16; i++) {
+                    const float re = __uint_as_float(rr[i]), im = __uint_as_float(ri[i]);
+                    if (16 * gg + i < kmax) prow[64 * (16 * gg + i)] = re * re + im * im;
+                }
+            }
+            if (++slot == 3) {
+                slot = 0;
+                u3++;
+            }
+        }
     }
     tc::fence_before_thread_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tD, TC_N);
+    if (tid == 0 && *abort_flag) atomicOr(status, FDAS_DEV_TIMEOUT);
+    if (warp == 0) {
+        tc::fence_after_thread_sync();
+        tc::tmem_dealloc(tbase, WS_TMEM_COLS);
+    }
 }
 
 }  // namespace
@@ -760,10 +914,8 @@ uint16_t host_bf16(float f) {
 }  // namespace
 
 // Host tables of the tensor path, FP64 then rounded once:
-//  - the split variant's F'[(k,p),(n,s)] (real-ified W_64^{kn}, re/im interleaved), K-major BF16
-//    images hi and lo;
 //  - F1 (stage 1: rows (p, k1), K in the stage-1 order) and F2 (stage 2: rows (p, k2), K = (s, n2)),
-//    K-major, in BF16 and in FP16;
+//    K-major, in BF16 (hi, and the rounding remainder lo of the split variant) and in FP16;
 //  - the four-step twiddles W_4096^{n2 k1}, [k1][n2].
 // Entry (p, s) of the real-ified W_64^{kn}: [[Re w, -Im w], [Im w, Re w]].
 static double dft64_real(int k, int n, int p, int s) {
@@ -777,31 +929,22 @@ static double dft64_real(int k, int n, int p, int s) {
 cudaError_t launch_prepare_bf16(Plan &p, cudaStream_t st) {
     const size_t T = (size_t)TC_M * TC_K;
     std::vector<uint16_t> img(4 * T, 0), img_h(2 * T, 0);
-    auto put = [&](size_t tile, int row, int k, double v) {
+    auto put = [&](size_t tile, int row, int k, double v) {       // tiles F1, F2, then their remainders
         const uint32_t o = tc::kmajor_offset(TC_M, row, k) / 2;
-        img[tile * T + o] = host_bf16((float)v);
-        if (tile >= 2) {
-            const __half h = __float2half_rn((float)v);
-            std::memcpy(&img_h[(tile - 2) * T + o], &h, 2);
-        }
+        const uint16_t b = host_bf16((float)v);
+        const uint32_t hb = (uint32_t)b << 16;
+        float hf;
+        std::memcpy(&hf, &hb, 4);
+        img[tile * T + o] = b;
+        img[(2 + tile) * T + o] = host_bf16((float)(v - (double)hf));
+        const __half h = __float2half_rn((float)v);
+        std::memcpy(&img_h[tile * T + o], &h, 2);
     };
-    for (int k = 0; k < TC_R; k++)
-        for (int n = 0; n < TC_R; n++)
-            for (int pr = 0; pr < 2; pr++)
-                for (int sg = 0; sg < 2; sg++) {
-                    const double v = dft64_real(k, n, pr, sg);
-                    const uint32_t o = tc::kmajor_offset(TC_M, 2 * k + pr, 2 * n + sg) / 2;
-                    img[o] = host_bf16((float)v);
-                    uint32_t hb = (uint32_t)img[o] << 16;
-                    float hf;
-                    std::memcpy(&hf, &hb, 4);
-                    img[T + o] = host_bf16((float)(v - (double)hf));
-                }
     for (int pr = 0; pr < 2; pr++)
         for (int k = 0; k < TC_R; k++)
             for (int kk = 0; kk < TC_K; kk++) {
-                put(2, TC_R * pr + k, kk, dft64_real(k, s1_n1(kk), pr, s1_s(kk)));     // F1
-                put(3, TC_R * pr + k, kk, dft64_real(k, kk & 63, pr, kk >> 6));         // F2
+                put(0, TC_R * pr + k, kk, dft64_real(k, s1_n1(kk), pr, s1_s(kk)));     // F1
+                put(1, TC_R * pr + k, kk, dft64_real(k, kk & 63, pr, kk >> 6));         // F2
             }
     std::vector<float2> tw(TC_R * TC_R);
     for (int k1 = 0; k1 < TC_R; k1++)
@@ -820,16 +963,16 @@ cudaError_t launch_prepare_bf16(Plan &p, cudaStream_t st) {
     return e;
 }
 
-// The register hand-over inside k3_plane_tc (setmaxnreg) assumes the launch allocation the kernel
+// The register hand-over inside the plane kernels (setmaxnreg) assumes the launch allocation the kernel
 // was compiled for; a different one could leave the increasing warps waiting, so it is checked
 // before every launch.
-template <class Ops>
-static cudaError_t prepare_plane_tc() {
+template <typename Kernel>
+static cudaError_t prepare_ws(Kernel kernel, uint32_t smem) {
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, k3_plane_tc<Ops>);
+    cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
     if (e != cudaSuccess) return e;
     if (fa.numRegs != REG_LAUNCH) return cudaErrorInvalidDeviceFunction;
-    return cudaFuncSetAttribute(k3_plane_tc<Ops>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)WS_SMEM);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
 static_assert(PEAK_CHUNK == 512, "the level-1 marks index units as bin >> 9");
@@ -852,7 +995,7 @@ cudaError_t launch_plane_bf16(const Plan &p, const float2 *d_x, const float *d_s
     const size_t smem2 = sizeof(float2) * fft_smem_entries(TC_S_BF16);
     cudaError_t e = cudaFuncSetAttribute(k2_segments_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
     if (e != cudaSuccess) return e;
-    e = prepare_plane_tc<OpsBF16>();
+    e = prepare_ws(k3_plane_tc<OpsBF16>, WS_SMEM);
     if (e != cudaSuccess) return e;
     // the unit marks are cleared by the segment kernel: their workspace slot is 256-byte aligned
     // and padded to 256 bytes, so whole 16-byte words cover it
@@ -872,7 +1015,7 @@ cudaError_t launch_plane_bf16(const Plan &p, const float2 *d_x, const float *d_s
     const int64_t grid = (n_items + per - 1) / per;
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
     k3_plane_tc<OpsBF16><<<(unsigned)grid, WS_THREADS, WS_SMEM, st>>>(
-        Y, reinterpret_cast<const uint4 *>(p.d_Gbf), reinterpret_cast<const uint4 *>(p.d_tcF) + 2 * TILE_BYTES / 16,
+        Y, reinterpret_cast<const uint4 *>(p.d_Gbf), reinterpret_cast<const uint4 *>(p.d_tcF),
         p.d_tcTw, d_plane, p.K, p.nb, p.L, n_items, n_groups, per, nullptr, l1flag, p.nb / PEAK_CHUNK, mark_threshold(p),
         p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
@@ -889,7 +1032,7 @@ cudaError_t launch_plane_f16(const Plan &p, const float2 *d_x, const float *d_sc
     const size_t smem2 = sizeof(float2) * fft_smem_entries(TC_S_BF16);
     cudaError_t e = cudaFuncSetAttribute(k2_segments_f16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
     if (e != cudaSuccess) return e;
-    e = prepare_plane_tc<OpsF16>();
+    e = prepare_ws(k3_plane_tc<OpsF16>, WS_SMEM);
     if (e != cudaSuccess) return e;
     p.prof.begin(FDAS_STAGE_SEGMENTS, st);
     k2_segments_f16<<<(unsigned)p.n_seg, TC_S_BF16 / 32, smem2, st>>>(d_x, d_scale, p.d_tw, Y, unscale,
@@ -927,18 +1070,17 @@ cudaError_t launch_plane_split(const Plan &p, const float2 *d_x, const float *d_
     // FP32 segment spectra (4096-bin CUDA-core block FFT), then the compensated tensor stages
     cudaError_t e = launch_segments_fp32(p, d_x, d_scale, Y, st);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k3_plane_tc_split, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SP_SMEM);
+    e = prepare_ws(k3_plane_tc_split, SP_SMEM);
     if (e != cudaSuccess) return e;
     const int n_groups = (p.K + TC_G - 1) / TC_G;
     const int64_t n_items = p.n_seg * n_groups;
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device >= 0 ? p.device : 0);
-    const int64_t ctas = std::min<int64_t>(n_items, (int64_t)sms * (p.tune_cta_per_sm > 0 ? p.tune_cta_per_sm : 1));
+    const int64_t ctas = std::min<int64_t>(n_items, (int64_t)sms);
     const int64_t per = (n_items + ctas - 1) / ctas;
     const int64_t grid = (n_items + per - 1) / per;
-    const uint4 *F = reinterpret_cast<const uint4 *>(p.d_tcF);
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    k3_plane_tc_split<<<(unsigned)grid, SP_THREADS, SP_SMEM, st>>>(Y, p.d_G, F, F + TILE_BYTES / 16, p.d_tcTw,
+    k3_plane_tc_split<<<(unsigned)grid, WS_THREADS, SP_SMEM, st>>>(Y, p.d_G, reinterpret_cast<const uint4 *>(p.d_tcF), p.d_tcTw,
                                                                    d_plane, p.K, p.nb, p.L, n_items, n_groups, per,
                                                                    p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
