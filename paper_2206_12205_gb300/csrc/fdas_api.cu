@@ -64,7 +64,7 @@ cudaError_t launch_plane_any(const Plan &p, const float2 *x, const float *scale,
         case FDAS_BF16_SPLIT: return launch_plane_split(p, x, scale, ws, static_cast<float *>(d_plane), st);
         case FDAS_FP16_SCALED: return launch_plane_f16(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag);
         case FDAS_BF16_DIRECT:
-            return launch_plane_direct(p, x, scale, ws, static_cast<__nv_bfloat16 *>(d_plane), st, l1flag);
+            return launch_plane_direct(p, x, scale, static_cast<__nv_bfloat16 *>(d_plane), st, l1flag);
         case FDAS_FP8_DIRECT: return launch_plane_direct_f8(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag);
         default: return launch_plane_fp32(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag);
     }
@@ -159,11 +159,9 @@ fdas_status fdas_plan(const fdas_config *cfg, fdas_plan_t *plan, size_t *workspa
         delete p;
         return FDAS_E_UNSUPPORTED;
     }
-    // segment spectra, or the BF16 direct path's packed spectrum (the FP8 direct path reads the
-    // spectrum itself)
-    const size_t ybytes = c.precision == FDAS_BF16_DIRECT ? sizeof(uint32_t) * fdas::direct_pack_words(*p)
-                          : c.precision == FDAS_FP8_DIRECT ? 256
-                                                           : sizeof(float2) * (size_t)p->n_seg * p->S;
+    // segment spectra (the direct paths read the spectrum itself)
+    const bool direct = c.precision == FDAS_BF16_DIRECT || c.precision == FDAS_FP8_DIRECT;
+    const size_t ybytes = direct ? 256 : sizeof(float2) * (size_t)p->n_seg * p->S;
     p->ws_y = off;     off = align_up(off + ybytes);
     p->ws_segscale = off; off = align_up(off + sizeof(float) * (size_t)p->n_seg);
     // the non-empty unit list directly before the counts (the kernels find it from the counts)

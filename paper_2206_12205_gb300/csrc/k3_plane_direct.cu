@@ -16,10 +16,19 @@
 // copies of its spectrum window in shared memory, shifted by b words so every descriptor starts
 // on a 16-byte boundary; the four MMA sets of a tile cover its 512 bins.
 //
-// One persistent CTA per SM (10 warps): warp 0 issues the MMAs (converged, elect.sync), warp 1
-// copies the windows, warps 2-9 read the accumulators (TMEM lanes = a, columns = (p, z)), form
-// |.|^2 and store the BF16 plane.  Two accumulator slots in TMEM, two window slots in shared
-// memory, every mbarrier wait bounded (timeout -> FDAS_DEV_TIMEOUT, MMAs drained, TMEM freed).
+// One persistent CTA per SM (12 warps): warp 0 issues the MMAs (converged, elect.sync), warps 1-3
+// make the windows (FP32 spectrum read once, scaled and rounded to BF16, each thread four words of
+// every copy with one 16-byte store per copy; the next tile's loads are in flight while the slot is
+// waited for), warps 4-11 read the accumulators (TMEM lanes = a, columns = (p, z)) and form |.|^2.
+// A lane's rows in the four sets of a tile are four consecutive bins, so its powers stay in
+// registers as BF16 pairs until the fourth set and leave as one 8-byte store per template: a warp
+// writes 256 consecutive bytes where one 2-byte store per set touched every sector four times.
+// Two accumulator slots in TMEM, two window slots in shared memory, every mbarrier wait bounded
+// (timeout -> FDAS_DEV_TIMEOUT, MMAs drained, TMEM freed).
+// The MMAs are its floor: each reads 4 KB of window and 16 N bytes of taps from shared memory (the
+// operand rate is 128 bytes a cycle), 4 m / 8 of them a tile.  N = 2^22, 21 templates, 64 taps: 95 us
+// and a separate packing pass of 8 us -> 55 us (before: one window warp on dependent 4-byte loads,
+// 2-byte stores 8 bytes apart).
 #include <cuda_fp8.h>
 
 #include "fdas_internal.cuh"
@@ -30,8 +39,9 @@ namespace fdas {
 namespace {
 
 constexpr int DT = 512;                          // bins per tile (4 sets x 128 rows)
-constexpr int D_WARPS = 10;
-constexpr int D_EPI0 = 2;                        // first epilogue warp
+constexpr int D_WARPS = 12;
+constexpr int D_WIN0 = 1, D_WIN = 3;             // window warps
+constexpr int D_EPI0 = 4;                        // first epilogue warp (a multiple of 4: TMEM lane quarters)
 constexpr long long D_WAIT = 4000000000LL;       // about 2 s at 2 GHz
 constexpr uint32_t D_MIN_SMEM = 120 * 1024;      // keeps one CTA (and one TMEM allocation) per SM
 
@@ -62,20 +72,16 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
                  : "r"(taddr));
 }
 
-// Xb[k] = Xhat[k - m/2] as a BF16 pair (zero outside the spectrum), k < n_out.
-__global__ void k3d_pack(const float2 *__restrict__ X, const float *__restrict__ scale_ptr, uint32_t *__restrict__ Xb,
-                         int64_t nb, int half_m, int64_t n_out) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n_out) return;
-    const float sc = scale_ptr ? __ldg(scale_ptr) : 1.0f;
-    const int64_t s = k - half_m;
-    float2 v = make_float2(0.f, 0.f);
-    if (s >= 0 && s < nb) v = __ldg(X + s);
-    const __nv_bfloat162 h = __floats2bfloat162_rn(v.x * sc, v.y * sc);
-    Xb[k] = *reinterpret_cast<const uint32_t *>(&h);
+__device__ __forceinline__ uint32_t d_pack(float lo, float hi) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&h);
 }
 
-__global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct(const uint32_t *__restrict__ Xb,
+// KHM: the most templates an epilogue warp holds (Kpad / 2 rounded up to 16, 32 or 64), which sets
+// the registers of its BF16 pairs.
+template <int KHM>
+__global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct(const float2 *__restrict__ X,
+                                                                   const float *__restrict__ scale_ptr,
                                                                    const uint4 *__restrict__ Bimg,
                                                                    __nv_bfloat16 *__restrict__ plane, int K, int Kpad,
                                                                    int m, int64_t nb, int64_t n_tiles,
@@ -98,7 +104,7 @@ __global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct(const uint32_
     }
     if (tid == 0) {
         for (int s = 0; s < 2; s++) {
-            tc::mbar_init(&bars->w_full[s], 32);
+            tc::mbar_init(&bars->w_full[s], 32 * D_WIN);
             tc::mbar_init(&bars->w_free[s], 1);
             tc::mbar_init(&bars->d_full[s], 1);
             tc::mbar_init(&bars->d_free[s], 256);
@@ -149,72 +155,153 @@ __global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct(const uint32_
             tc::mbar_wait_bounded(&bars->drain, 0, D_WAIT);
         }
         __syncwarp();
-    } else if (warp == 1) {
-        // ---------------------------------------------------------------- window copies
-        // copy b of slot s holds Xb[r0 + b + j], j < WW (the rows r0 + 4 a + b, a < 128, read
-        // Xb[r0 + 4 a + b + q], q < m)
-        for (int64_t k = 0; k < n_my; k++) {
-            if (k >= 2 && !d_wait(&bars->w_free[k & 1], (uint32_t)(((k - 2) >> 1) & 1), abort_flag)) break;
-            const int64_t r0 = (t0 + k) * DT;
-            uint32_t *dst = sW + (size_t)(k & 1) * 4 * WW;
-#pragma unroll 1
-            for (int b = 0; b < 4; b++)
-                for (int j = lane; j < WW; j += 32) dst[b * WW + j] = __ldg(Xb + r0 + b + j);
-            tc::fence_proxy_async_smem();
-            d_arrive(&bars->w_full[k & 1]);
+    } else if (warp < D_EPI0) {
+        // ---------------------------------------------------------------- windows
+        // word w of the tile's window is Xhat[r0 + w - m/2] (zero outside the spectrum); copy b holds
+        // the words b .. WW + b - 1 (the rows r0 + 4 a + b, a < 128, read words 4 a + b + q, q < m).
+        // A thread takes the words 4 i .. 4 i + 3 and, from its neighbour, the next three.
+        const float sc = scale_ptr ? __ldg(scale_ptr) : 1.0f;
+        // The loads run two steps (a step: 96 threads, one pass of a tile) ahead of their use.
+        const int groups = WW / 4;
+        constexpr int T = 32 * D_WIN;
+        const int t = tid - 32 * D_WIN0, passes = (groups + T - 1) / T;
+        const int64_t steps = n_my * passes;
+        struct Words {
+            float2 v[7];
+        };
+        auto load = [&](int64_t k, int p) {
+            Words w;
+            const int i = t + p * T;
+            const int64_t r = (t0 + k) * DT - m / 2 + 4 * i;
+            const int need = i >= groups ? 0 : (lane == 31 || i == groups - 1) ? 7 : 4;   // no neighbour: all seven
+#pragma unroll
+            for (int j = 0; j < 7; j++) {
+                w.v[j] = make_float2(0.f, 0.f);
+                if (j < need && r + j >= 0 && r + j < nb) w.v[j] = __ldg(X + r + j);
+            }
+            return w;
+        };
+        auto put = [&](const Words &in, int64_t k, int p) {
+            const int i = t + p * T;
+            uint32_t w[7];
+#pragma unroll
+            for (int j = 0; j < 7; j++) w[j] = d_pack(in.v[j].x * sc, in.v[j].y * sc);
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                const uint32_t next = __shfl_down_sync(0xffffffffu, w[j], 1);
+                if (lane != 31 && i != groups - 1) w[4 + j] = next;
+            }
+            if (i < groups) {
+                uint32_t *dst = sW + (size_t)(k & 1) * 4 * WW + 4 * i;
+#pragma unroll
+                for (int b = 0; b < 4; b++)
+                    *reinterpret_cast<uint4 *>(dst + b * WW) = make_uint4(w[b], w[b + 1], w[b + 2], w[b + 3]);
+            }
+        };
+        Words ahead[2];
+        int64_t kl = 0;                                    // tile and pass of the next load
+        int pl = 0;
+        auto advance = [&](int64_t &k, int &p) {
+            if (++p == passes) {
+                p = 0;
+                k++;
+            }
+        };
+#pragma unroll
+        for (int e = 0; e < 2; e++) {
+            if (e < steps) ahead[e] = load(kl, pl);
+            advance(kl, pl);
+        }
+        int64_t k = 0;
+        int p = 0;
+        bool ok = true;
+        for (int64_t s = 0; s < steps && ok; s += 2) {
+#pragma unroll
+            for (int e = 0; e < 2; e++) {
+                if (s + e >= steps) break;
+                if (p == 0 && k >= 2) {
+                    ok = d_wait(&bars->w_free[k & 1], (uint32_t)(((k - 2) >> 1) & 1), abort_flag);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                }
+                put(ahead[e], k, p);
+                if (s + e + 2 < steps) ahead[e] = load(kl, pl);
+                advance(kl, pl);
+                if (p == passes - 1) {
+                    tc::fence_proxy_async_smem();
+                    d_arrive(&bars->w_full[k & 1]);
+                }
+                advance(k, p);
+            }
         }
     } else {
         // ---------------------------------------------------------------- epilogue
-        // thread -> TMEM lane a (row r = r0 + 4 a + b), templates z in [h Kh, h Kh + Kh)
+        // thread -> TMEM lane a (bins r0 + 4 a + b), templates z in [h Kh, h Kh + Kh)
         const int quad = warp & 3, h = (warp - D_EPI0) >> 2;
-        const int a = 32 * quad + lane, Kh = Kpad / 2;
+        const int a = 32 * quad + lane, Kh = Kpad / 2;      // Kh: a multiple of 4, at most KHM
+        const int z_lo = h * Kh, z_n = min(Kh, K - z_lo);   // templates stored
         const uint32_t lane_base = (uint32_t)(32 * quad) << 16;
         for (int64_t k = 0; k < n_my; k++) {
-            const int64_t r0 = (t0 + k) * DT;
+            const int64_t r = (t0 + k) * DT + 4 * a;
             bool ok = true;
+            // pw[b / 2][z]: the power of set b (even b: FP32, until the odd set completes the BF16 pair)
+            uint32_t pw[2][KHM];
+#pragma unroll
             for (int b = 0; b < 4; b++) {
                 const int64_t u = 4 * k + b;
-                const int sl = (int)(u & 1);
-                if (!d_wait(&bars->d_full[sl], (uint32_t)((u >> 1) & 1), abort_flag)) {
-                    ok = false;
-                    break;
-                }
+                const int sl = b & 1;
+                if (ok && !d_wait(&bars->d_full[sl], (uint32_t)((u >> 1) & 1), abort_flag)) ok = false;
+                if (!ok) break;
                 tc::fence_after_thread_sync();
-                const int64_t r = r0 + 4 * a + b;
-                const bool in = r < nb;
-                const uint32_t col = tbase + lane_base + (uint32_t)sl * N;
-                for (int z0 = h * Kh; z0 < h * Kh + Kh; z0 += 4) {
-                    uint32_t re[4], im[4];
-                    tmem_ld4(col + z0, re);
-                    tmem_ld4(col + Kpad + z0, im);
-                    tc::tmem_ld_wait();
-                    if (z0 + 4 >= h * Kh + Kh) {                 // the slot's last read: release it
-                        tc::fence_before_thread_sync();
-                        d_arrive(&bars->d_free[sl]);
-                    }
-                    if (in) {
-                        float vs[4];
+                const uint32_t col = tbase + lane_base + (uint32_t)sl * N + z_lo;
 #pragma unroll
-                        for (int e = 0; e < 4; e++) {
-                            const int z = z0 + e;
-                            vs[e] = -INFINITY;
-                            if (z < K) {
-                                const float xr = __uint_as_float(re[e]), xi = __uint_as_float(im[e]);
-                                const __nv_bfloat16 v = __float2bfloat16_rn(xr * xr + xi * xi);
-                                plane[(int64_t)z * nb + r] = v;
-                                vs[e] = __bfloat162float(v);
-                            }
+                for (int c = 0; c < KHM; c += 8) {
+                    if (c < Kh) {                            // warp-uniform
+                        uint32_t re[2][4], im[2][4];
+                        tmem_ld4(col + c, re[0]);
+                        tmem_ld4(col + Kpad + c, im[0]);
+                        if (c + 4 < Kh) {
+                            tmem_ld4(col + c + 4, re[1]);
+                            tmem_ld4(col + Kpad + c + 4, im[1]);
                         }
-                        // level-1 marks of the units (z, r / 512) whose stored value is above thr1 (rare)
-                        if (l1flag != nullptr && fmaxf(fmaxf(vs[0], vs[1]), fmaxf(vs[2], vs[3])) > thr1) {
+                        tc::tmem_ld_wait();
 #pragma unroll
-                            for (int e = 0; e < 4; e++)
-                                if (vs[e] > thr1) l1flag[(int64_t)(z0 + e) * chunks1 + (r >> 9)] = 1;
+                        for (int e = 0; e < 8; e++) {
+                            if (e >= 4 && c + 4 >= Kh) break;
+                            const float xr = __uint_as_float(re[e >> 2][e & 3]), xi = __uint_as_float(im[e >> 2][e & 3]);
+                            const float p = xr * xr + xi * xi;
+                            pw[b >> 1][c + e] = (b & 1) ? d_pack(__uint_as_float(pw[b >> 1][c + e]), p) : __float_as_uint(p);
+                        }
+                    }
+                }
+                tc::fence_before_thread_sync();              // the slot is drained
+                d_arrive(&bars->d_free[sl]);
+            }
+            if (!ok) break;
+            if (r < nb) {
+                __nv_bfloat16 *row = plane + (int64_t)z_lo * nb + r;
+                __nv_bfloat162 top = __floats2bfloat162_rn(0.f, 0.f);    // powers are not negative
+#pragma unroll
+                for (int z = 0; z < KHM; z++) {
+                    if (z < z_n) {
+                        *reinterpret_cast<uint2 *>(row + (int64_t)z * nb) = make_uint2(pw[0][z], pw[1][z]);
+                        top = __hmax2(top, __hmax2(*reinterpret_cast<__nv_bfloat162 *>(&pw[0][z]),
+                                                   *reinterpret_cast<__nv_bfloat162 *>(&pw[1][z])));
+                    }
+                }
+                // level-1 marks of the units (z, r / 512) whose stored value is above thr1 (rare)
+                if (l1flag != nullptr && fmaxf(__low2float(top), __high2float(top)) > thr1) {
+#pragma unroll
+                    for (int z = 0; z < KHM; z++) {
+                        if (z < z_n) {
+                            const __nv_bfloat162 q = __hmax2(*reinterpret_cast<__nv_bfloat162 *>(&pw[0][z]),
+                                                             *reinterpret_cast<__nv_bfloat162 *>(&pw[1][z]));
+                            if (fmaxf(__low2float(q), __high2float(q)) > thr1)
+                                l1flag[(int64_t)(z_lo + z) * chunks1 + (r >> 9)] = 1;
                         }
                     }
                 }
             }
-            if (!ok) break;
         }
     }
     tc::fence_before_thread_sync();
@@ -248,6 +335,7 @@ __global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct(const uint32_
 // templates each) and store the plane.  Every wait is bounded (FDAS_DEV_TIMEOUT), copies in
 // flight are awaited and TMEM is freed before exit.
 constexpr int DT8 = 1024;
+constexpr int D8_WARPS = 10, D8_EPI0 = 2;        // warps, first epilogue warp
 constexpr int F8_TPG = 32;                       // templates per group (N = 64)
 constexpr int F8_N = 2 * F8_TPG;
 
@@ -279,7 +367,7 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
                  : "memory");
 }
 
-__global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct_f8(const float2 *__restrict__ X,
+__global__ void __launch_bounds__(D8_WARPS * 32, 1) k3_plane_direct_f8(const float2 *__restrict__ X,
                                                                       const float *__restrict__ scale_ptr,
                                                                       const uint4 *__restrict__ Bimg,
                                                                       const float *__restrict__ tsig,
@@ -320,7 +408,7 @@ __global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct_f8(const floa
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (uint32_t i = tid; i < b_bytes / 16; i += D_WARPS * 32) reinterpret_cast<uint4 *>(sB)[i] = __ldg(Bimg + i);
+    for (uint32_t i = tid; i < b_bytes / 16; i += D8_WARPS * 32) reinterpret_cast<uint4 *>(sB)[i] = __ldg(Bimg + i);
     tc::fence_proxy_async_smem();
     tc::fence_before_thread_sync();
     __syncthreads();
@@ -434,7 +522,7 @@ __global__ void __launch_bounds__(D_WARPS * 32, 1) k3_plane_direct_f8(const floa
             tc::mbar_wait_bounded(&bars->raw_full[k & 1], (uint32_t)((k >> 1) & 1), D_WAIT);
     } else {
         // ------------------------------------------------------------------ epilogue
-        const int quad = warp & 3, h = (warp - D_EPI0) >> 2;
+        const int quad = warp & 3, h = (warp - D8_EPI0) >> 2;
         const int a = 32 * quad + lane;
         const uint32_t lane_base = (uint32_t)(32 * quad) << 16;
         bool ok = true;
@@ -537,7 +625,7 @@ cudaError_t launch_plane_direct_f8(const Plan &p, const float2 *d_x, const float
     const int64_t per = (n_tiles + ctas - 1) / ctas;
     const int64_t grid = (n_tiles + per - 1) / per;
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    k3_plane_direct_f8<<<(unsigned)grid, D_WARPS * 32, smem, st>>>(d_x, d_scale, reinterpret_cast<const uint4 *>(p.d_dimg),
+    k3_plane_direct_f8<<<(unsigned)grid, D8_WARPS * 32, smem, st>>>(d_x, d_scale, reinterpret_cast<const uint4 *>(p.d_dimg),
                                                                    p.d_dsig, d_plane, p.K, G, p.m, p.nb, n_tiles, per,
                                                                    l1flag, p.nb / PEAK_CHUNK, mark_threshold(p), p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
@@ -560,24 +648,10 @@ bool direct_geometry(const Plan &p, int *Kpad, uint32_t *smem_bytes, uint32_t *t
     return true;
 }
 
-size_t direct_pack_words(const Plan &p) {
-    const int64_t n_tiles = (p.nb + DT - 1) / DT;
-    return (size_t)(n_tiles * DT + p.m + 4);
-}
-
-cudaError_t launch_plane_direct(const Plan &p, const float2 *d_x, const float *d_scale, char *ws,
-                                __nv_bfloat16 *d_plane, cudaStream_t st, uint8_t *l1flag) {
-    int Kpad = 0;
-    uint32_t smem = 0, cols = 0;
-    if (!p.d_dimg || !direct_geometry(p, &Kpad, &smem, &cols)) return cudaErrorInvalidValue;
-    uint32_t *Xb = reinterpret_cast<uint32_t *>(ws + p.ws_y);
-    const int64_t n_out = (int64_t)direct_pack_words(p);
-    p.prof.begin(FDAS_STAGE_SEGMENTS, st);
-    k3d_pack<<<(unsigned)((n_out + 255) / 256), 256, 0, st>>>(d_x, d_scale, Xb, p.nb, p.m / 2, n_out);
-    p.prof.end(FDAS_STAGE_SEGMENTS, st);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k3_plane_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+template <int KHM>
+static cudaError_t run_direct(const Plan &p, const float2 *d_x, const float *d_scale, __nv_bfloat16 *d_plane, cudaStream_t st,
+                              uint8_t *l1flag, int Kpad, uint32_t smem, uint32_t cols) {
+    cudaError_t e = cudaFuncSetAttribute(k3_plane_direct<KHM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (l1flag) {
         e = cudaMemsetAsync(l1flag, 0, (size_t)p.K * (size_t)(p.nb / PEAK_CHUNK), st);
@@ -590,12 +664,22 @@ cudaError_t launch_plane_direct(const Plan &p, const float2 *d_x, const float *d
     const int64_t per = (n_tiles + ctas - 1) / ctas;
     const int64_t grid = (n_tiles + per - 1) / per;
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    k3_plane_direct<<<(unsigned)grid, D_WARPS * 32, smem, st>>>(Xb, reinterpret_cast<const uint4 *>(p.d_dimg), d_plane,
-                                                                p.K, Kpad, p.m, p.nb, n_tiles, per, cols, l1flag,
-                                                                p.nb / PEAK_CHUNK, mark_threshold(p), p.d_status);
+    k3_plane_direct<KHM><<<(unsigned)grid, D_WARPS * 32, smem, st>>>(
+        d_x, d_scale, reinterpret_cast<const uint4 *>(p.d_dimg), d_plane, p.K, Kpad, p.m, p.nb, n_tiles, per, cols, l1flag,
+        p.nb / PEAK_CHUNK, mark_threshold(p), p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
-    p.prof.launches += 2;
+    p.prof.launches += 1;
     return cudaGetLastError();
+}
+
+cudaError_t launch_plane_direct(const Plan &p, const float2 *d_x, const float *d_scale, __nv_bfloat16 *d_plane,
+                                cudaStream_t st, uint8_t *l1flag) {
+    int Kpad = 0;
+    uint32_t smem = 0, cols = 0;
+    if (!p.d_dimg || !direct_geometry(p, &Kpad, &smem, &cols)) return cudaErrorInvalidValue;
+    if (Kpad <= 32) return run_direct<16>(p, d_x, d_scale, d_plane, st, l1flag, Kpad, smem, cols);
+    if (Kpad <= 64) return run_direct<32>(p, d_x, d_scale, d_plane, st, l1flag, Kpad, smem, cols);
+    return run_direct<64>(p, d_x, d_scale, d_plane, st, l1flag, Kpad, smem, cols);
 }
 
 }  // namespace fdas
