@@ -195,37 +195,45 @@ __global__ void k1_apply_scale(const float2 *__restrict__ X, const float *__rest
 // sqrt(2 ln 2 / med_b), med_b = the lower median (rank floor((n - 1) / 2) in ascending order) of
 // |X_k|^2 over the block's n bins with k >= 1.  For noise |X_k|^2 is exponential, whose median is
 // its mean times ln 2, so the normalised noise power has mean 2 in every block; a median is not
-// moved by the few bins a signal occupies.  One CTA per block: the powers are sorted in shared
-// memory (bitonic, the excluded DC bin as +inf) and the rank picked exactly.
-__global__ void __launch_bounds__(256) k1_local_norm(const float2 *__restrict__ X, float2 *__restrict__ out, int B) {
-    extern __shared__ float pw[];
+// moved by the few bins a signal occupies.  One CTA per block, the powers in registers (the excluded
+// DC bin as +inf).  Non-negative floats order like their bits, so the rank is found bit by bit from
+// the top: the median's next bit is set when no more than `rank` values lie below the prefix with
+// it set.  31 counts of the block's values, each a compare per value and one barrier, in place of
+// the 78 compare-exchange passes of a bitonic sort of 4096 powers through shared memory: N = 2^21,
+// blocks of 4096: 43 -> 8 us.
+template <int PER>
+__global__ void __launch_bounds__(1024) k1_local_norm(const float2 *__restrict__ X, float2 *__restrict__ out, int B) {
+    __shared__ int part[2][32];
+    const int T = blockDim.x, t = threadIdx.x, lane = t & 31, warps = T >> 5;
     const int64_t k0 = (int64_t)blockIdx.x * B;
-    for (int i = threadIdx.x; i < B; i += 256) {
-        const float2 v = X[k0 + i];
-        pw[i] = (k0 + i == 0) ? INFINITY : v.x * v.x + v.y * v.y;
-    }
-    __syncthreads();
-    for (int size = 2; size <= B; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < B / 2; i += 256) {
-                const int lo = 2 * i - (i & (stride - 1));          // first of the pair
-                const int hi = lo + stride;
-                const bool up = (lo & size) == 0;
-                const float a = pw[lo], b = pw[hi];
-                if ((a > b) == up) {
-                    pw[lo] = b;
-                    pw[hi] = a;
-                }
-            }
-            __syncthreads();
-        }
+    uint32_t pw[PER];
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const float2 v = X[k0 + t + i * T];
+        const float p = __fmaf_rn(v.y, v.y, __fmul_rn(v.x, v.x));
+        pw[i] = (k0 + t + i * T == 0) ? 0x7f800000u : __float_as_uint(p);
     }
     const int n = (k0 == 0) ? B - 1 : B;
-    const float med = pw[(n - 1) / 2];
-    const float s = med > 0.f ? sqrtf(2.0f * 0.69314718f / med) : 0.f;
-    for (int i = threadIdx.x; i < B; i += 256) {
-        const float2 v = X[k0 + i];
-        out[k0 + i] = make_float2(v.x * s, v.y * s);
+    const int rank = (n - 1) / 2;
+    uint32_t med = 0;
+    for (int bit = 30; bit >= 0; bit--) {
+        const uint32_t trial = med | (1u << bit);
+        int below = 0;
+#pragma unroll
+        for (int i = 0; i < PER; i++) below += pw[i] < trial;
+        below = __reduce_add_sync(0xffffffffu, below);
+        if (lane == 0) part[bit & 1][t >> 5] = below;
+        __syncthreads();                              // the two halves of `part` alternate
+        below = __reduce_add_sync(0xffffffffu, lane < warps ? part[bit & 1][lane] : 0);
+        if (below <= rank) med = trial;
+    }
+    const float m = __uint_as_float(med);
+    const float s = m > 0.f ? sqrtf(2.0f * 0.69314718f / m) : 0.f;
+#pragma unroll
+    for (int i = 0; i < PER; i++) {
+        const int64_t k = k0 + t + i * T;
+        const float2 v = X[k];
+        out[k] = make_float2(v.x * s, v.y * s);
     }
 }
 
@@ -300,12 +308,16 @@ cudaError_t launch_spectrum(const Plan &p, const float *d_series, char *ws, cuda
 cudaError_t launch_local_norm(const Plan &p, const float2 *d_x, float2 *d_out, cudaStream_t st) {
     const int B = p.cfg.norm_block;
     if (B <= 0 || p.nb % B != 0) return cudaErrorInvalidValue;
-    if (B * sizeof(float) > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k1_local_norm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)(B * sizeof(float)));
-        if (e != cudaSuccess) return e;
+    // 16 values a thread between 512 and 16384 bins (fewer, larger blocks of threads outside)
+    const unsigned blocks = (unsigned)(p.nb / B);
+    switch (B) {
+        case 64: k1_local_norm<2><<<blocks, 32, 0, st>>>(d_x, d_out, B); break;
+        case 128: k1_local_norm<4><<<blocks, 32, 0, st>>>(d_x, d_out, B); break;
+        case 256: k1_local_norm<8><<<blocks, 32, 0, st>>>(d_x, d_out, B); break;
+        case 32768: k1_local_norm<32><<<blocks, 1024, 0, st>>>(d_x, d_out, B); break;
+        case 65536: k1_local_norm<64><<<blocks, 1024, 0, st>>>(d_x, d_out, B); break;
+        default: k1_local_norm<16><<<blocks, B / 16, 0, st>>>(d_x, d_out, B); break;
     }
-    k1_local_norm<<<(unsigned)(p.nb / B), 256, B * sizeof(float), st>>>(d_x, d_out, B);
     p.prof.launches += 1;
     return cudaGetLastError();
 }
