@@ -170,7 +170,9 @@ fdas_status fdas_plan(const fdas_config *cfg, fdas_plan_t *plan, size_t *workspa
     p->ws_umask = off;  off = align_up(off + sizeof(uint32_t) * (fdas::PEAK_CHUNK / 32) * (size_t)p->n_units);
     p->ws_l1flag = off; off = align_up(off + (size_t)p->K * (size_t)(p->nb / fdas::PEAK_CHUNK));
     // the level search's work list (the entries of its block order that are not skipped)
-    p->ws_k4work = off; off = align_up(off + sizeof(uint32_t) * (size_t)std::max<int64_t>(1, fdas::levels_order_size(*p)));
+    // followed by a bit per entry of the order
+    const int64_t n_order = fdas::levels_order_size(*p);
+    p->ws_k4work = off; off = align_up(off + sizeof(uint32_t) * (size_t)(std::max<int64_t>(1, n_order) + (n_order + 31) / 32));
     p->ws_bytes = off;
     p->device = -1;
     *plan = p;

@@ -101,11 +101,12 @@ struct Plan {
 // (level, row, chunk) with a count and a PEAK_CHUNK-bit mask.
 constexpr int PEAK_ROWS = 8;
 constexpr int PEAK_CHUNK = 512;
-// The non-empty peak units, listed as the level kernels count them: a 4-word header (the list's
-// count, then the level search's work count) and up to PEAK_LIST_CAP unit numbers, placed in the
-// workspace directly before the unit counts.  When the list holds them all, the output block
-// orders and emits them; else it scans every unit's count.
-constexpr int PEAK_LIST_CAP = 1024;
+// The peak units with cells above their threshold, listed as the level kernels find them: a 4-word
+// header (the list's count, then the level search's work count) and up to PEAK_LIST_CAP unit numbers,
+// placed in the workspace directly before the unit counts.  When the list holds them all, the output
+// blocks share the listed units; else they scan every unit's count.  4096: the list and its counts
+// fill 32 KB of an output block's shared memory, and summing it per unit still costs a warp under 1 us.
+constexpr int PEAK_LIST_CAP = 4096;
 constexpr int PEAK_LIST_WORDS = 4 + PEAK_LIST_CAP;
 
 struct LevelDesc {

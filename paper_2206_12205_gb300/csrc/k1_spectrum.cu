@@ -200,7 +200,7 @@ __global__ void k1_apply_scale(const float2 *__restrict__ X, const float *__rest
 // the top: the median's next bit is set when no more than `rank` values lie below the prefix with
 // it set.  31 counts of the block's values, each a compare per value and one barrier, in place of
 // the 78 compare-exchange passes of a bitonic sort of 4096 powers through shared memory: N = 2^21,
-// blocks of 4096: 43 -> 8 us.
+// blocks of 4096: 43 -> 13 us.
 template <int PER>
 __global__ void __launch_bounds__(1024) k1_local_norm(const float2 *__restrict__ X, float2 *__restrict__ out, int B) {
     __shared__ int part[2][32];

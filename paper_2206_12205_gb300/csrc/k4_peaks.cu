@@ -17,16 +17,22 @@
 // r0 + l + 32 e, e < 16 -- so that one warp-wide load of harmonic h reads 32 elements h apart,
 // a span of whole sectors, where consecutive bins per lane would touch 32 sectors per load.  A
 // lane tests its 16 values against the threshold through their maximum; only cells above it (a
-// handful per plane) recompute their 3x3 neighbourhood's sums to decide the peak.
+// handful per plane, thousands with low thresholds) recompute their 3x3 neighbourhood's sums to
+// decide the peak: nine lanes of a warp to a cell (verify_unit), from the mask of such cells that the
+// level kernels leave; on BF16 planes level 1 and the plain sums' levels decide theirs in place
+// (IN_PLACE: what each way costs).
 //
 // Output order (H, i, r): a "unit" is (level, row, chunk of CB bins), units are numbered in
 // that order, and
-//   pass A (k4_level1 over the plane, k4_levels over level 2's region) writes each unit's peak
-//     count and, when non-zero, its CB-bit mask, and lists the non-empty units (in no order);
-//   pass B (k4_emit_listed, one block): when the list holds every non-empty unit (PEAK_LIST_CAP;
-//     the usual case) it sorts the list's unit numbers, scans their counts into offsets and
-//     writes the records; otherwise it scans every unit's count in order.  Either way a
-//     record's power is S_H recomputed at its cell, at offset + rank.
+//   pass A (k4_level1 over the plane, k4_levels over level 2's region, then k4_verify where cells
+//     were left to it) writes each unit's peak count and, when cells were above the threshold, its
+//     CB-bit mask, and lists those units (in no order);
+//   pass B (k4_emit_listed): when the list holds all of them (PEAK_LIST_CAP; the usual case) each
+//     listed unit goes to a warp, which sums the counts of the units before it and writes its
+//     records; otherwise every unit's count is scanned in order.  Either way a record's power is
+//     S_H recomputed at its cell, at offset + rank.
+// Listed calls with thousands of peaks (FP32 plane, N = 2^21, 85 templates, low thresholds, some 3000
+// units): 260 -> 139 us, of which the tests were 50 and the output 75.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -163,10 +169,13 @@ template <typename E>
 __device__ __forceinline__ float harm_sum(const E *plane, int64_t nb, int zmax, int H, int i, int64_t r) {
     const int z = -zmax + 2 * i;
     float s = 0.0f;
-    for (int h = 1; h <= H; h++) {
-        const int ih = (h * z + zmax) >> 1;
-        s = __fadd_rn(s, ld_plane(plane, (int64_t)ih * nb + (int64_t)h * r));
-    }
+    float v[16];                                         // all the gathers in flight together
+#pragma unroll
+    for (int h = 1; h <= 16; h++)
+        if (h <= H) v[h - 1] = ld_plane(plane, (int64_t)((h * z + zmax) >> 1) * nb + (int64_t)h * r);
+#pragma unroll
+    for (int h = 1; h <= 16; h++)
+        if (h <= H) s = __fadd_rn(s, v[h - 1]);
     return s;
 }
 
@@ -179,13 +188,18 @@ template <typename E>
 __device__ float harm_sum_anch(const E *plane, int64_t nb, int zmax, int H, int i, int64_t r) {
     const int z = -zmax + 2 * i;
     float s = ld_plane(plane, (int64_t)i * nb + r);
-    for (int l = 1; (1 << l) <= H; l++) {
+#pragma unroll
+    for (int l = 1; l <= 4; l++) {                       // a level's loads (at most 8) in flight together
         const int L = 1 << l;
+        if (L > H) break;
+        float v[8];
+#pragma unroll
         for (int j = 1; j < L; j += 2) {
             const int ij = (j * z + L * zmax + L) >> (l + 1);
-            const int64_t rj = (2 * (int64_t)j * r + L) >> (l + 1);
-            s = __fadd_rn(s, ld_plane(plane, (int64_t)ij * nb + rj));
+            v[j >> 1] = ld_plane(plane, (int64_t)ij * nb + ((2 * (int64_t)j * r + L) >> (l + 1)));
         }
+#pragma unroll
+        for (int j = 1; j < L; j += 2) s = __fadd_rn(s, v[j >> 1]);
     }
     return s;
 }
@@ -231,19 +245,32 @@ __device__ __forceinline__ void add_level(const E *__restrict__ plane, int64_t n
     }
 }
 
-// The 3x3 rule for a cell of level H holding S_H = v: strictly above the defined neighbours that
-// come earlier in row-major (i, r) order, at least equal to the later ones.
+// harm_sum with U gathers in flight.
+template <typename E, int U = 2>
+__device__ __forceinline__ float harm_sum_inorder(const E *plane, int64_t nb, int zmax, int H, int i, int64_t r) {
+    const int z = -zmax + 2 * i;
+    float s = 0.0f;
+#pragma unroll U
+    for (int h = 1; h <= H; h++)
+        s = __fadd_rn(s, ld_plane(plane, (int64_t)((h * z + zmax) >> 1) * nb + (int64_t)h * r));
+    return s;
+}
+
+// The 3x3 rule for a cell of level H holding S_H = v, by one lane inside the level search: strictly
+// above the defined neighbours that come earlier in row-major (i, r) order, at least equal to the
+// later ones.  The registers it asks for are the caller's loss: with its sums' gathers unrolled by
+// the compiler's choice the search spilled, and N = 2^23, BF16, took 207 us instead of 191 (all 16 in
+// flight: 275).
 template <typename E>
-__device__ __noinline__ bool local_max(const E *plane, int64_t nb, int zmax, int K, int H, int64_t rmax, int i, int64_t r, float v,
-                                       bool anchored = false) {
+__device__ __noinline__ bool local_max(const E *plane, int64_t nb, int zmax, int K, int H, int64_t rmax, int i, int64_t r, float v) {
     for (int di = -1; di <= 1; di++) {
         const int ii = i + di;
-        if (anchored ? (ii < 0 || ii >= K) : !row_in_level(ii, K, zmax, H)) continue;
+        if (!row_in_level(ii, K, zmax, H)) continue;
         for (int dr = -1; dr <= 1; dr++) {
             if (di == 0 && dr == 0) continue;
             const int64_t rr = r + dr;
             if (rr < 0 || rr > rmax) continue;
-            const float w = anchored ? harm_sum_anch(plane, nb, zmax, H, ii, rr) : harm_sum(plane, nb, zmax, H, ii, rr);
+            const float w = harm_sum_inorder(plane, nb, zmax, H, ii, rr);
             const bool earlier = di < 0 || (di == 0 && dr < 0);
             if (earlier ? !(v > w) : !(v >= w)) return false;
         }
@@ -259,58 +286,115 @@ __device__ __forceinline__ unsigned int *unit_list(int32_t *unit_count) {
 __device__ __forceinline__ const unsigned int *unit_list(const int32_t *unit_count) {
     return reinterpret_cast<const unsigned int *>(unit_count) - PEAK_LIST_WORDS;
 }
-// A unit's count, and the unit on the list when it holds peaks (one thread per unit; the list
-// append, a handful of times per plane, out of line so that it costs the callers no registers).
+// The unit on the list (one thread per unit; out of line, a handful of times per plane, so that it
+// costs the callers no registers).
 __device__ __noinline__ void list_unit(int32_t *unit_count, int64_t u) {
     unsigned int *list = unit_list(unit_count);
     const unsigned int slot = atomicAdd(list, 1u);
     if (slot < (unsigned int)PEAK_LIST_CAP) list[4 + slot] = (unsigned int)u;
 }
+
+// A unit's count, and the unit on the list when it holds peaks (one thread per unit).
 __device__ __forceinline__ void count_unit(int32_t *__restrict__ unit_count, int64_t u, int cnt) {
     unit_count[u] = cnt;
     if (cnt > 0) list_unit(unit_count, u);
 }
 
-// One level H > 1 of one (row, chunk), lane bins rb + 32 e: S_H from S_{H/2}, then the unit's count
-// and mask (word e of the mask, bins 32 e .. 32 e + 31 of the chunk, is the warp's ballot of bit e).
-// Returns false when the chunk lies outside level H's region (the regions nest: stop there).
+// Whether the plain sums' level search (k4_levels*) tests its cells in place instead of leaving them to
+// k4_verify.  N = 2^23, 85 templates, the whole region: BF16 planes 191 us in place, 253 us leaving
+// them; FP32 planes 229 us in place, 209 us leaving them (the compiler schedules the kernels' loads
+// differently).  FP32, N = 2^21 with low thresholds, thousands of cells to test: 130 us in place, 63 us.
+template <typename E>
+constexpr bool IN_PLACE = sizeof(E) == 2;
+
+// What the level kernels leave of one unit u to be tested: a zero count, or, when a cell is above the
+// threshold, the mask of those cells, the unit on the list and a count of -1.  word: lane w < 16 holds
+// word w of the mask, bins 32 w .. 32 w + 31.
+__device__ __forceinline__ void leave_unit(uint32_t word, int u, int32_t *__restrict__ unit_count,
+                                           uint32_t *__restrict__ unit_mask) {
+    const int lane = threadIdx.x & 31;
+    if (lane < WORDS) unit_mask[(int64_t)u * WORDS + lane] = word;
+    if (lane == 0) {
+        unit_count[u] = -1;
+        list_unit(unit_count, u);
+    }
+}
+
+// The same from a warp's sums: s[e] of bin lane + 32 e, bins defined up to rest.
+__device__ __forceinline__ void leave_sums(const float (&s)[LB], float thr, int rest, int u, int32_t *__restrict__ unit_count,
+                                           uint32_t *__restrict__ unit_mask) {
+    const int lane = threadIdx.x & 31;
+    float vmax = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < LB; e++)
+        if (lane + 32 * e <= rest) vmax = fmaxf(vmax, s[e]);
+    if (__any_sync(0xffffffffu, vmax > thr)) {
+        uint32_t word = 0;
+#pragma unroll
+        for (int e = 0; e < LB; e++) {
+            const uint32_t b = __ballot_sync(0xffffffffu, lane + 32 * e <= rest && s[e] > thr);
+            if (lane == e) word = b;
+        }
+        leave_unit(word, u, unit_count, unit_mask);
+    } else if (lane == 0) {
+        unit_count[u] = 0;
+    }
+}
+
+// The same from a lane's 16 consecutive bins (bit e of above: bin 16 lane + e).
+__device__ __forceinline__ void leave_runs(uint32_t above, int u, int32_t *__restrict__ unit_count,
+                                           uint32_t *__restrict__ unit_mask) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t lo = __shfl_sync(0xffffffffu, above, (2 * lane) & 31), hi = __shfl_sync(0xffffffffu, above, (2 * lane + 1) & 31);
+    if (__any_sync(0xffffffffu, above != 0)) leave_unit(lo | (hi << 16), u, unit_count, unit_mask);
+    else if (lane == 0) unit_count[u] = 0;
+}
+
+// One level H > 1 of one (row, chunk), lane bins rb + 32 e: S_H from S_{H/2}, then the unit's peaks or
+// its cells above the threshold (word e of the mask, bins 32 e .. 32 e + 31 of the chunk, is the
+// warp's ballot of bit e).  Returns false when the chunk lies outside level H's region (the regions
+// nest: stop there).
 template <typename E, int H, bool ADD = true>
 __device__ __forceinline__ bool level_step(const E *__restrict__ plane, int64_t nb, int zmax, int K,
                                            const LevelDesc &d, int i, int z, int chunk, int64_t rb, float (&s)[LB],
                                            int32_t *__restrict__ unit_count, uint32_t *__restrict__ unit_mask) {
-    const int lane = threadIdx.x & 31;
     if (!row_in_level(i, K, zmax, H) || (int64_t)chunk * CB > d.rmax) return false;   // warp-uniform
     if (ADD) add_level<E, H>(plane, nb, zmax, z, rb, d.rmax, s);
-    float vmax = -INFINITY;
-#pragma unroll
-    for (int e = 0; e < LB; e++)
-        if (rb + 32 * e <= d.rmax) vmax = fmaxf(vmax, s[e]);
     // unit indices fit 32 bits (at most 1023 rows x 2^17 chunks per level, five levels)
     const int u = (int)d.unit0 + (i - d.i_lo) * (int)d.chunks + chunk;
-    if (__any_sync(0xffffffffu, vmax > d.thr)) {
-        uint32_t pk = 0;
-        if (vmax > d.thr) {
+    if constexpr (IN_PLACE<E>) {
+        const int lane = threadIdx.x & 31;
+        float vmax = -INFINITY;
 #pragma unroll
-            for (int e = 0; e < LB; e++) {
-                const int64_t r = rb + 32 * e;
-                if (r <= d.rmax && s[e] > d.thr && local_max(plane, nb, zmax, K, H, d.rmax, i, r, s[e])) pk |= 1u << e;
+        for (int e = 0; e < LB; e++)
+            if (rb + 32 * e <= d.rmax) vmax = fmaxf(vmax, s[e]);
+        if (__any_sync(0xffffffffu, vmax > d.thr)) {
+            uint32_t pk = 0;
+            if (vmax > d.thr) {
+#pragma unroll
+                for (int e = 0; e < LB; e++) {
+                    const int64_t r = rb + 32 * e;
+                    if (r <= d.rmax && s[e] > d.thr && local_max(plane, nb, zmax, K, H, d.rmax, i, r, s[e])) pk |= 1u << e;
+                }
             }
-        }
-        int cnt = __popc(pk);
+            int cnt = __popc(pk);
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        if (lane == 0) count_unit(unit_count, u, cnt);
-        if (cnt > 0) {
-            uint32_t word = 0;
+            for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+            if (lane == 0) count_unit(unit_count, u, cnt);
+            if (cnt > 0) {
+                uint32_t word = 0;
 #pragma unroll
-            for (int e = 0; e < LB; e++) {
-                const uint32_t b = __ballot_sync(0xffffffffu, (pk >> e) & 1u);
-                if (lane == e) word = b;
+                for (int e = 0; e < LB; e++) {
+                    const uint32_t b = __ballot_sync(0xffffffffu, (pk >> e) & 1u);
+                    if (lane == e) word = b;
+                }
+                if (lane < WORDS) unit_mask[(int64_t)u * WORDS + lane] = word;
             }
-            if (lane < WORDS) unit_mask[(int64_t)u * WORDS + lane] = word;
+        } else if (lane == 0) {
+            unit_count[u] = 0;
         }
-    } else if (lane == 0) {
-        unit_count[u] = 0;
+    } else {
+        leave_sums(s, d.thr, (int)min(d.rmax - (int64_t)chunk * CB, (int64_t)CB), u, unit_count, unit_mask);
     }
     return true;
 }
@@ -348,17 +432,168 @@ __device__ __forceinline__ void detect_chunk(const E *__restrict__ plane, int64_
     }
 }
 
-// The level-1 peaks among a lane's 16 bins rl .. rl + 15 of row i (a lane holding a value above
-// the threshold, a handful per plane): re-read, test each against the 3x3 rule, return the mask.
+struct UnitRef {
+    int H, row;
+    int64_t chunk, rmax;
+};
+
+// Level, row and chunk of unit u (selects, not an indexed table: that would sit in local memory).
+__device__ __forceinline__ UnitRef unit_of(const LevelTable &lt, int64_t u) {
+    UnitRef ref;
+    ref.H = 1;
+    ref.rmax = lt.lev[0].rmax;
+    int i_lo = lt.lev[0].i_lo;
+    int64_t local = u, chunks = lt.lev[0].chunks;
+#pragma unroll
+    for (int k = 1; k < 5; k++)
+        if (k < lt.n_levels && u >= lt.lev[k].unit0) {
+            ref.H = lt.lev[k].H;
+            ref.rmax = lt.lev[k].rmax;
+            i_lo = lt.lev[k].i_lo;
+            local = u - lt.lev[k].unit0;
+            chunks = lt.lev[k].chunks;
+        }
+    // unit numbers and chunk counts fit 32 bits
+    const uint32_t q = (uint32_t)local / (uint32_t)chunks;
+    ref.row = i_lo + (int)q;
+    ref.chunk = (uint32_t)local - q * (uint32_t)chunks;
+    return ref;
+}
+
+// The mask of a unit's peaks (lane w < 16: word w) among its cells when they are many: a lane to a bin,
+// 32 consecutive bins at a time, so that the gathers of a warp share their sectors.  Every lane's own
+// sum serves its row neighbours through shuffles; then the cells still standing look at the rows
+// before and after, each lane up to the first neighbour that beats its cell.  With every second cell of
+// an FP32 plane above the threshold (N = 2^23, 54 million peaks) the whole call takes 19.8 ms, in place
+// 20.3 and nine lanes to a cell 71.
 template <typename E>
-__device__ __noinline__ uint32_t level1_peaks(const E *__restrict__ plane, int64_t nb, int zmax, int K,
-                                              const LevelDesc d, int i, int64_t rl) {
-    uint32_t pk = 0;
-    for (int e = 0; e < LB; e++) {
-        const float v = ld_plane(plane, (int64_t)i * nb + rl + e);
-        if (v > d.thr && local_max(plane, nb, zmax, K, 1, d.rmax, i, rl + e, v)) pk |= 1u << e;
+__device__ __noinline__ uint32_t verify_dense(const E *__restrict__ plane, int64_t nb, int zmax, int K, bool anchored, int H,
+                                              int row, int64_t r0, int64_t rmax, uint32_t cells) {
+    const int lane = threadIdx.x & 31;
+    uint32_t word = 0;
+    for (int e = 0; e < WORDS; e++) {
+        const uint32_t bits = __shfl_sync(0xffffffffu, cells, e);
+        if (bits == 0) continue;                     // warp-uniform
+        const int64_t r = r0 + 32 * e + lane;
+        bool ok = (bits >> lane) & 1u;
+        float v = 0.0f, edge = 0.0f;                 // S(row, r); lanes 0 and 31: S of the bin before and after
+        // k = 0: the own sums, 1: the edges', 2 .. 7: the other rows' (one copy of the sums' code)
+#pragma unroll 1
+        for (int k = 0; k < 8; k++) {
+            const int a = k < 2 ? 0 : k < 5 ? -1 : 1, d = k == 0 ? 0 : k == 1 ? (lane == 0 ? -1 : 1) : (k - 2) % 3 - 1;
+            const int ii = row + a;
+            const int64_t rr = r + d;
+            const bool defined = (anchored ? (ii >= 0 && ii < K) : row_in_level(ii, K, zmax, H)) && rr >= 0 && rr <= rmax;
+            const bool want = defined && (k == 0 || (ok && (k > 1 || lane == 0 || lane == 31)));
+            float w = 0.0f;
+            if (want) w = anchored ? harm_sum_anch(plane, nb, zmax, H, ii, rr) : harm_sum_inorder<E, 4>(plane, nb, zmax, H, ii, rr);
+            if (k == 0) {
+                v = w;
+            } else if (k == 1) {
+                edge = w;
+                const float before = __shfl_up_sync(0xffffffffu, v, 1), after = __shfl_down_sync(0xffffffffu, v, 1);
+                if (r > 0 && !(v > (lane == 0 ? edge : before))) ok = false;
+                if (r < rmax && !(v >= (lane == 31 ? edge : after))) ok = false;
+                if (!__any_sync(0xffffffffu, ok)) break;
+            } else if (want) {
+                ok = a < 0 ? v > w : v >= w;
+            }
+        }
+        const uint32_t b = __ballot_sync(0xffffffffu, ok);
+        if (lane == e) word = b;
     }
-    return pk;
+    return word;
+}
+
+// The peaks of one unit u among the cells its mask holds: its count and the mask of the peaks.  The
+// 3x3 rule for a cell: strictly above the defined neighbours that come earlier in row-major (i, r)
+// order, at least equal to the later ones.
+// One warp, nine lanes to a cell, three cells at a time, each lane one of the nine sums with its
+// gathers in flight together: one or two round trips to L2 per three cells.  (One lane per cell, its
+// neighbours one after another, cost up to 8 H dependent round trips for each cell of a lane, and the
+// cells along a strong signal were often all in one lane.)  From DENSE_CELLS cells on the
+// gathers' sectors cost more than their latency: verify_dense (FP32, N = 2^23, 11 million peaks, mostly
+// units of 30 to 200 cells: 12 ms with the line at 32, 6.6 at 128, 6.0 at 256; in place 12.4).
+constexpr int DENSE_CELLS = 256;
+template <typename E>
+__device__ __forceinline__ void verify_unit(const E *__restrict__ plane, int64_t nb, int zmax, int K, bool anchored,
+                                            const UnitRef &ref, int64_t u, int32_t *__restrict__ unit_count,
+                                            uint32_t *__restrict__ unit_mask) {
+    const int lane = threadIdx.x & 31, H = ref.H;
+    const uint32_t cells = lane < WORDS ? unit_mask[u * WORDS + lane] : 0u;
+    int incl = __popc(cells);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const int g = lane / 9, q = lane - 9 * g, a = q / 3 - 1, d = q % 3 - 1;          // cell of three, neighbour
+    const int ii = ref.row + a;
+    const bool row_ok = anchored ? (ii >= 0 && ii < K) : row_in_level(ii, K, zmax, H);
+    uint32_t word = 0;                               // lane w < 16: word w of the peaks' mask
+    const int listed = total < DENSE_CELLS ? total : 0;
+    if (listed < total) word = verify_dense<E>(plane, nb, zmax, K, anchored, H, ref.row, ref.chunk * CB, ref.rmax, cells);
+    for (int k0 = 0; k0 < listed; k0 += 3) {         // warp-uniform
+        const int k = k0 + g;                        // the group's cell: the first word with incl > k holds it
+        int w = 0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, incl, w + o - 1) <= k) w += o;
+        const int last = __shfl_sync(0xffffffffu, incl, w);
+        uint32_t bits = __shfl_sync(0xffffffffu, cells, w);
+        const bool live = g < 3 && k < total;
+        int bin = 0;
+        bool ok = false;
+        float sum = 0.0f;
+        if (live) {
+            for (int skip = k - (last - __popc(bits)); skip > 0; skip--) bits &= bits - 1;
+            bin = 32 * w + __ffs(bits) - 1;
+            const int64_t r = ref.chunk * CB + bin + d;
+            ok = row_ok && r >= 0 && r <= ref.rmax;
+            if (ok) sum = anchored ? harm_sum_anch(plane, nb, zmax, H, ii, r) : harm_sum(plane, nb, zmax, H, ii, r);
+        }
+        const float v = __shfl_sync(0xffffffffu, sum, (9 * g + 4) & 31);
+        const uint32_t beaten = __ballot_sync(0xffffffffu, ok && q != 4 && !(q < 4 ? v > sum : v >= sum));
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            const int b = __shfl_sync(0xffffffffu, bin, 9 * c + 4);
+            if (k0 + c < total && !(beaten & (0x1ffu << (9 * c))) && lane == (b >> 5)) word |= 1u << (b & 31);
+        }
+    }
+    int cnt = __popc(word);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    if (lane == 0) unit_count[u] = cnt;
+    if (lane < WORDS) unit_mask[u * WORDS + lane] = word;
+}
+
+// One level-1 unit u of row i, bins r0 .. r0 + 511, that holds a value above the threshold: its cells,
+// and, where nothing else needs k4_verify (IN_PLACE), its peaks.  Out of line, the values read again, so
+// that the stream over the plane keeps its registers.
+template <typename E>
+__device__ __noinline__ void level1_unit(const E *__restrict__ plane, int64_t nb, int zmax, int K, const LevelDesc &d, int i,
+                                         int64_t r0, int u, bool in_place, int32_t *__restrict__ unit_count,
+                                         uint32_t *__restrict__ unit_mask) {
+    typename Fmt<E>::Raw raw;
+    Fmt<E>::load_raw(plane + (int64_t)i * nb + r0 + LB * (threadIdx.x & 31), raw);
+    float v[LB];
+    Fmt<E>::widen(raw, v);
+    uint32_t above = 0;
+#pragma unroll
+    for (int e = 0; e < LB; e++)
+        if (v[e] > d.thr) above |= 1u << e;
+    leave_runs(above, u, unit_count, unit_mask);
+    // many cells: here, while the rows around are in the caches
+    if ((in_place && __any_sync(0xffffffffu, above != 0)) || (int)__reduce_add_sync(0xffffffffu, __popc(above)) >= DENSE_CELLS) {
+        __syncwarp();                                // the mask and the count of leave_runs, then their rewrite
+        UnitRef ref;
+        ref.H = 1;
+        ref.row = i;
+        ref.chunk = r0 / CB;
+        ref.rmax = d.rmax;
+        verify_unit<E>(plane, nb, zmax, K, false, ref, u, unit_count, unit_mask);
+    }
 }
 
 // Level 1 over the whole plane: a pure stream.  Grid (ceil(chunks1 / (DETECT_WARPS * CPW1)), K);
@@ -367,7 +602,7 @@ __device__ __noinline__ uint32_t level1_peaks(const E *__restrict__ plane, int64
 // candidate.  Few registers, so many warps keep the loads in flight.
 template <typename E>
 __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_L1_MIN_BLOCKS) k4_level1(const E *__restrict__ plane, int64_t nb, int zmax,
-                                                              int K, LevelDesc d, int chunks1,
+                                                              int K, LevelDesc d, int chunks1, bool in_place,
                                                               int32_t *__restrict__ unit_count,
                                                               uint32_t *__restrict__ unit_mask) {
     constexpr int CPW1 = Fmt<E>::EPV == 8 ? 4 : 2;
@@ -380,23 +615,18 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_L1_MIN_BLOCKS) k4_l
 #pragma unroll
     for (int c = 0; c < CPW1; c++)
         if (c0 + c < chunks1) Fmt<E>::load_raw(row + (int64_t)(c0 + c) * CB + LB * lane, raw[c]);
+    uint32_t hot = 0;                                // the chunks with a value above the threshold
 #pragma unroll
     for (int c = 0; c < CPW1; c++) {
         if (c0 + c >= chunks1) break;
-        const float vmax = Fmt<E>::max16(raw[c]);
         const int u = (int)d.unit0 + i * (int)d.chunks + c0 + c;
-        if (__any_sync(0xffffffffu, vmax > d.thr)) {
-            const uint32_t pk =
-                vmax > d.thr ? level1_peaks(plane, nb, zmax, K, d, i, (int64_t)(c0 + c) * CB + LB * lane) : 0u;
-            int cnt = __popc(pk);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-            const uint32_t hi = __shfl_down_sync(0xffffffffu, pk, 1);
-            if (lane == 0) count_unit(unit_count, u, cnt);
-            if (cnt > 0 && !(lane & 1)) unit_mask[(int64_t)u * WORDS + (lane >> 1)] = pk | (hi << 16);
-        } else if (lane == 0) {
-            unit_count[u] = 0;
-        }
+        if (__any_sync(0xffffffffu, Fmt<E>::max16(raw[c]) > d.thr)) hot |= 1u << c;
+        else if (lane == 0) unit_count[u] = 0;
+    }
+    for (; hot; hot &= hot - 1) {
+        const int c = c0 + __ffs(hot) - 1;
+        level1_unit<E>(plane, nb, zmax, K, d, i, (int64_t)c * CB, (int)d.unit0 + i * (int)d.chunks + c, in_place, unit_count,
+                       unit_mask);
     }
 }
 
@@ -413,13 +643,14 @@ __device__ __forceinline__ bool chunk_needs_search(const uint8_t *__restrict__ m
 
 // The level search's work list: one thread per entry k of the block order (row << 16 | 4-chunk
 // group); an entry is kept when any of its chunks needs the search (chunk_needs_search), else its
-// chunks' level-2 units count zero here.  Kept entries are appended per warp in the order's order
-// (ballot prefix, one atomic per warp), so the list keeps the ray order's locality; *count
-// (word 1 of the unit list's header) was cleared before the peak search.  Whole warps call it.
+// chunks' level-2 units count zero here.  Whole warps call it.  Short orders: kept entries are appended
+// per warp (ballot prefix, one atomic; *count, word 1 of the unit list's header, was cleared before the
+// peak search), in whatever order the warps come by.  Long ones (keep != nullptr): the warp leaves its
+// ballot, and k4_compact writes the list in the order's order, on which the search's locality rests.
 __device__ __noinline__ void select_entry(int64_t k, const uint32_t *__restrict__ order, int64_t n_order,
                                              const uint8_t *__restrict__ marks, int zmax, int K, const LevelTable &lt,
                                              int chunks2, uint32_t *__restrict__ work, unsigned int *__restrict__ count,
-                                             int32_t *__restrict__ unit_count) {
+                                             uint32_t *__restrict__ keep_words, int32_t *__restrict__ unit_count) {
     const int lane = threadIdx.x & 31;
     bool keep = false;
     uint32_t o = 0;
@@ -438,10 +669,42 @@ __device__ __noinline__ void select_entry(int64_t k, const uint32_t *__restrict_
         }
     }
     const uint32_t b = __ballot_sync(0xffffffffu, keep);
+    if (keep_words != nullptr) {
+        if (lane == 0 && k < n_order) keep_words[k >> 5] = b;
+        return;
+    }
     unsigned int base = 0;
     if (lane == 0 && b) base = atomicAdd(count, (unsigned int)__popc(b));
     base = __shfl_sync(0xffffffffu, base, 0);
     if (keep) work[base + __popc(b & ((1u << lane) - 1u))] = o;
+}
+
+// The work list of a long order from the warps' ballots (keep, one word per 32 entries): a block takes
+// eight words, counts the entries kept before them (a few KB from L2) and writes its own in order.
+// Appended as the warps came by, the list was in random order (mean displacement 4000 of 13887) and
+// the search had lost the ray order's locality: N = 2^23, 85 templates, BF16.
+__global__ void __launch_bounds__(256) k4_compact(const uint32_t *__restrict__ keep, const uint32_t *__restrict__ order,
+                                                  int64_t n_order, uint32_t *__restrict__ work, unsigned int *__restrict__ count) {
+    __shared__ unsigned int before[8], own[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t n_words = (n_order + 31) / 32, w0 = 8 * (int64_t)blockIdx.x, w = w0 + warp;
+    unsigned int sum = 0;
+    for (int64_t i = threadIdx.x; i < w0; i += 256) sum += __popc(keep[i]);
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    const uint32_t bits = w < n_words ? keep[w] : 0u;
+    if (lane == 0) {
+        before[warp] = sum;
+        own[warp] = __popc(bits);
+    }
+    __syncthreads();
+    unsigned int base = 0, total = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++) {
+        base += before[i] + (i < warp ? own[i] : 0u);
+        total += before[i] + own[i];
+    }
+    if ((bits >> lane) & 1u) work[base + __popc(bits & ((1u << lane) - 1u))] = order[32 * w + lane];
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *count = total;
 }
 
 // Level 1 after a plane kernel that marked its units (flags[u] != 0: the unit u = i chunks + c holds
@@ -452,17 +715,18 @@ __device__ __noinline__ void select_entry(int64_t k, const uint32_t *__restrict_
 // thread per entry of the block order; n_order = 0: none): the list depends only on the marks.
 template <typename E>
 __global__ void __launch_bounds__(DETECT_WARPS * 32) k4_level1_marked(const E *__restrict__ plane, int64_t nb, int zmax,
-                                                                    int K, LevelDesc d, int64_t n_units1,
+                                                                    int K, LevelDesc d, bool in_place, int64_t n_units1,
                                                                     const uint8_t *__restrict__ flags,
                                                                     int32_t *__restrict__ unit_count,
                                                                     uint32_t *__restrict__ unit_mask,
                                                                     int64_t l1_blocks,
                                                                     const uint32_t *__restrict__ order, int64_t n_order,
-                                                                    LevelTable lt, int chunks2, uint32_t *__restrict__ work) {
+                                                                    LevelTable lt, int chunks2, uint32_t *__restrict__ work,
+                                                                    uint32_t *__restrict__ keep) {
     const int lane = threadIdx.x & 31;
     if (blockIdx.x >= l1_blocks) {                   // block-uniform
         select_entry((int64_t)(blockIdx.x - l1_blocks) * blockDim.x + threadIdx.x, order, n_order, flags, zmax, K, lt,
-                     chunks2, work, unit_list(unit_count) + 1, unit_count);
+                     chunks2, work, unit_list(unit_count) + 1, keep, unit_count);
         return;
     }
     const int64_t u0 = ((int64_t)blockIdx.x * DETECT_WARPS + (threadIdx.x >> 5)) * 32;
@@ -475,16 +739,8 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32) k4_level1_marked(const E *_
         const int64_t uu = u0 + (__ffs(todo) - 1);
         todo &= todo - 1;
         const int i = (int)(uu / d.chunks);
-        const int64_t rl = (uu - (int64_t)i * d.chunks) * CB + LB * lane;
-        typename Fmt<E>::Raw raw;
-        Fmt<E>::load_raw(plane + (int64_t)i * nb + rl, raw);
-        const uint32_t pk = Fmt<E>::max16(raw) > d.thr ? level1_peaks(plane, nb, zmax, K, d, i, rl) : 0u;
-        int cnt = __popc(pk);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        const uint32_t hi = __shfl_down_sync(0xffffffffu, pk, 1);
-        if (lane == 0) count_unit(unit_count, d.unit0 + uu, cnt);
-        if (cnt > 0 && !(lane & 1)) unit_mask[(d.unit0 + uu) * WORDS + (lane >> 1)] = pk | (hi << 16);
+        level1_unit<E>(plane, nb, zmax, K, d, i, (uu - (int64_t)i * d.chunks) * CB, (int)(d.unit0 + uu), in_place, unit_count,
+                       unit_mask);
     }
 }
 
@@ -626,40 +882,6 @@ __device__ __forceinline__ void anch_add_level(const E *__restrict__ plane, int6
     }
 }
 
-// The count and mask of one anchored unit (row i, chunk c) of level L, lane bins rb + 32 e.
-template <typename E>
-__device__ __forceinline__ void anch_unit(const E *__restrict__ plane, int64_t nb, int zmax, int K, const LevelDesc &d,
-                                          int L, int i, int c, int64_t rb, const float (&s)[LB],
-                                          int32_t *__restrict__ unit_count, uint32_t *__restrict__ unit_mask) {
-    const int lane = threadIdx.x & 31;
-    float vmax = s[0];
-#pragma unroll
-    for (int e = 1; e < LB; e++) vmax = fmaxf(vmax, s[e]);
-    const int u = (int)d.unit0 + i * (int)d.chunks + c;
-    if (__any_sync(0xffffffffu, vmax > d.thr)) {
-        uint32_t pk = 0;
-        if (vmax > d.thr) {
-            for (int e = 0; e < LB; e++)
-                if (s[e] > d.thr && local_max(plane, nb, zmax, K, L, d.rmax, i, rb + 32 * e, s[e], true)) pk |= 1u << e;
-        }
-        int cnt = __popc(pk);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        if (lane == 0) count_unit(unit_count, u, cnt);
-        if (cnt > 0) {
-            uint32_t word = 0;
-#pragma unroll
-            for (int e = 0; e < LB; e++) {
-                const uint32_t bal = __ballot_sync(0xffffffffu, (pk >> e) & 1u);
-                if (lane == e) word = bal;
-            }
-            if (lane < WORDS) unit_mask[(int64_t)u * WORDS + lane] = word;
-        }
-    } else if (lane == 0) {
-        unit_count[u] = 0;
-    }
-}
-
 // Levels 2 .. 16 of the anchored sums for one (row i, chunk c), lane bins rb + 32 e.
 template <typename E>
 __device__ __forceinline__ void anch_chunk(const E *__restrict__ plane, int64_t nb, int zmax, int K, const LevelTable &lt,
@@ -674,17 +896,20 @@ __device__ __forceinline__ void anch_chunk(const E *__restrict__ plane, int64_t 
 #pragma unroll
         for (int e = 0; e < LB; e++) s[e] = ld_plane(row, rb + 32 * e);
     }
+    auto leave = [&](int l) {                        // the anchored levels cover whole chunks of every row
+        leave_sums(s, lt.lev[l].thr, CB - 1, (int)lt.lev[l].unit0 + i * (int)lt.lev[l].chunks + c, unit_count, unit_mask);
+    };
     anch_add_level<E, 1>(plane, nb, zmax, z, (uint32_t)rb, s);
-    anch_unit<E>(plane, nb, zmax, K, lt.lev[1], 2, i, c, rb, s, unit_count, unit_mask);
+    leave(1);
     if (lt.n_levels < 3) return;
     anch_add_level<E, 2>(plane, nb, zmax, z, (uint32_t)rb, s);
-    anch_unit<E>(plane, nb, zmax, K, lt.lev[2], 4, i, c, rb, s, unit_count, unit_mask);
+    leave(2);
     if (lt.n_levels < 4) return;
     anch_add_level<E, 3>(plane, nb, zmax, z, (uint32_t)rb, s);
-    anch_unit<E>(plane, nb, zmax, K, lt.lev[3], 8, i, c, rb, s, unit_count, unit_mask);
+    leave(3);
     if (lt.n_levels < 5) return;
     anch_add_level<E, 4>(plane, nb, zmax, z, (uint32_t)rb, s);
-    anch_unit<E>(plane, nb, zmax, K, lt.lev[4], 16, i, c, rb, s, unit_count, unit_mask);
+    leave(4);
 }
 
 template <typename E>
@@ -713,34 +938,70 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_MIN_BLOCKS) k4a_lev
     anch_chunk<E>(plane, nb, zmax, K, lt, (int)(o >> 16), c, unit_count, unit_mask);
 }
 
-struct UnitRef {
-    int l, row;
-    int64_t chunk;
-};
-
-__device__ __forceinline__ UnitRef unit_of(const LevelTable &lt, int64_t u) {
-    int l = 0;
+// The units with cells above their threshold, one warp each: the listed ones, or, when they are more
+// than the list holds, every unit whose count is -1: level 1's in order, the others in the order of the
+// level search (order: entries row << 16 | chunk group, rows from lt.lev[1].i_lo; nullptr: column by
+// column), so that the sums around a unit's cells find their sectors in L2 (FP32, N = 2^23, 42 million
+// peaks: 37 ms in the units' order, 20 in the search's).  Four blocks to an SM at 64 registers: the
+// gathers' latency is hidden by warps (anchored sums, N = 2^21, 19 million peaks: 13.8 ms with two, 12.0).
+constexpr int VERIFY_WARPS = 8;
+template <typename E>
+__global__ void __launch_bounds__(VERIFY_WARPS * 32, 4) k4_verify(const E *__restrict__ plane, int64_t nb, int zmax, int K,
+                                                               LevelTable lt, const uint32_t *__restrict__ order,
+                                                               int64_t n_order, int32_t *__restrict__ unit_count,
+                                                               uint32_t *__restrict__ unit_mask) {
+    const unsigned int *list = unit_list(unit_count);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int n = (int)*list;
+    const bool anchored = lt.anchored != 0;
+    if (n <= PEAK_LIST_CAP) {
+        for (int k = (int)blockIdx.x + wid * (int)gridDim.x; k < n; k += VERIFY_WARPS * (int)gridDim.x) {
+            const int64_t u = list[4 + k];
+            if (unit_count[u] >= 0) continue;            // tested in place
+            verify_unit<E>(plane, nb, zmax, K, anchored, unit_of(lt, u), u, unit_count, unit_mask);
+        }
+        return;
+    }
+    const int64_t n1 = (int64_t)K * lt.lev[0].chunks, b1 = (n1 + 31) / 32;      // level 1: 32 units to a warp
+    const int group = anchored ? DETECT_WARPS : DETECT_WARPS * CPW;             // chunks of an order's entry
+    const int64_t total = b1 + n_order * group;
+    for (int64_t k = (int64_t)blockIdx.x * VERIFY_WARPS + wid; k < total; k += (int64_t)gridDim.x * VERIFY_WARPS) {
+        // the warp's up to 32 units, one per lane (level 1), or its chunk's levels 2 .. (lanes 1 .. 4)
+        int64_t u = -1;
+        if (k < b1) {
+            if (32 * k + lane < n1) u = 32 * k + lane;
+        } else if (lane > 0 && lane < lt.n_levels) {
+            const int64_t o = (k - b1) / group;
+            const uint32_t code = order ? __ldg(order + o) : (uint32_t)(o % lt.lev[1].rows) << 16 | (uint32_t)(o / lt.lev[1].rows);
+            const int i = lt.lev[1].i_lo + (int)(code >> 16), c = (int)(code & 0xffffu) * group + (int)((k - b1) % group);
+            int i_lo = 0, rows = 0;
+            int64_t unit0 = 0, chunks = 0;
 #pragma unroll
-    for (int k = 1; k < 5; k++)
-        if (k < lt.n_levels && u >= lt.lev[k].unit0) l = k;
-    const LevelDesc &d = lt.lev[l];
-    const int64_t local = u - d.unit0;
-    UnitRef ref;
-    ref.l = l;
-    ref.row = d.i_lo + (int)(local / d.chunks);
-    ref.chunk = local % d.chunks;
-    return ref;
+            for (int l = 1; l < 5; l++)
+                if (l == lane) {
+                    i_lo = lt.lev[l].i_lo;
+                    rows = lt.lev[l].rows;
+                    unit0 = lt.lev[l].unit0;
+                    chunks = lt.lev[l].chunks;
+                }
+            if (i >= i_lo && i < i_lo + rows && c < chunks) u = unit0 + (int64_t)(i - i_lo) * chunks + c;
+        }
+        uint32_t todo = __ballot_sync(0xffffffffu, u >= 0 && unit_count[u < 0 ? 0 : u] < 0);
+        for (; todo; todo &= todo - 1) {
+            const int64_t uu = __shfl_sync(0xffffffffu, u, __ffs(todo) - 1);
+            verify_unit<E>(plane, nb, zmax, K, anchored, unit_of(lt, uu), uu, unit_count, unit_mask);
+        }
+    }
 }
 
-// The records of one non-empty unit u, the first at out[base]: one warp, the unit's mask words
-// one per lane, the peaks in bin order (the order of the output within a unit).
+// The records of one non-empty unit u, the first at out[base]: one warp, the unit's mask words one
+// per lane, the peaks dealt to the lanes in bin order (the order of the output within a unit).
 template <typename E>
-__device__ __forceinline__ void emit_unit(const E *__restrict__ plane, int64_t nb, int zmax, const LevelTable &lt,
-                                          int64_t u, int64_t base, const uint32_t *__restrict__ unit_mask,
-                                          fdas_peak *__restrict__ out, int max_peaks, uint32_t series) {
+__device__ __noinline__ void emit_unit(const E *__restrict__ plane, int64_t nb, int zmax, bool anchored, UnitRef ref,
+                                       int64_t u, int64_t base, const uint32_t *__restrict__ unit_mask,
+                                       fdas_peak *__restrict__ out, int max_peaks, uint32_t series) {
     const int lane = threadIdx.x & 31;
-    const UnitRef ref = unit_of(lt, u);
-    const int H = lt.lev[ref.l].H;
+    const int H = ref.H;
     const uint32_t w = lane < WORDS ? unit_mask[u * WORDS + lane] : 0u;
     int incl = __popc(w);
 #pragma unroll
@@ -748,24 +1009,32 @@ __device__ __forceinline__ void emit_unit(const E *__restrict__ plane, int64_t n
         const int y = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += y;
     }
-    int64_t pos = base + incl - __popc(w);
-    uint32_t bits = w;
-    while (bits) {
-        const int b = __ffs(bits) - 1;
-        bits &= bits - 1;
-        if (pos < max_peaks) {
-            const int64_t r = ref.chunk * CB + lane * 32 + b;
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    for (int k0 = 0; k0 < total; k0 += 32) {                 // warp-uniform
+        const int k = k0 + lane;                             // this lane's peak of the unit
+        int word = 0, before = 0;
+#pragma unroll
+        for (int j = 0; j < WORDS; j++) {                    // the word holding it: the first with incl > k
+            const int ij = __shfl_sync(0xffffffffu, incl, j);
+            if (ij <= k) {
+                word = j + 1;
+                before = ij;
+            }
+        }
+        uint32_t bits = __shfl_sync(0xffffffffu, w, word & 31);
+        if (k < total && base + k < max_peaks) {
+            for (int skip = k - before; skip > 0; skip--) bits &= bits - 1;
+            const int64_t r = ref.chunk * CB + word * 32 + (__ffs(bits) - 1);
             fdas_peak pk;
             pk.series = series;
             pk.r = (uint32_t)r;
             pk.zi = (int16_t)ref.row;
             pk.harm = (uint8_t)H;
             pk.pad = 0;
-            pk.power = lt.anchored ? harm_sum_anch(plane, nb, zmax, H, ref.row, r)
+            pk.power = anchored ? harm_sum_anch(plane, nb, zmax, H, ref.row, r)
                                    : harm_sum(plane, nb, zmax, H, ref.row, r);
-            out[pos] = pk;
+            out[base + k] = pk;
         }
-        pos++;
     }
 }
 
@@ -798,23 +1067,25 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t c, int32_t *warp_tot,
 }
 
 // The step's peaks, blocks of 1024 threads.  Usually the non-empty unit list holds every
-// non-empty unit (a handful to a few hundred of ~10^6): block 0 alone sorts its unit numbers by
-// rank (they are distinct: rank = how many are smaller), scans their counts in that order into
-// output offsets and emits each unit's records with one warp; the other blocks return at once.
+// non-empty unit (a handful to a few thousand of ~10^6): unit k of the list goes to warp k / grid of
+// block k mod grid, which sums the counts of the listed units with smaller numbers (its output
+// offset; the list and its counts in shared memory, 32 a step) and emits the unit's records.
 // Units are numbered in (level, row, chunk) order, so the records come out in (H, i, r) order.
+// One block that sorted the list and emitted all units itself took 51 us for some 600 units of
+// anchored sums, this 6 us.
 // When more than PEAK_LIST_CAP units hold peaks (low thresholds, up to millions of peaks), every
 // block takes a contiguous range of units: it sums the counts before its range (its first output
 // offset; a few MB read from L2 per block, no communication between blocks), then scans its
 // range 4096 units a round and emits the non-empty units as it goes.  The last block (or block 0
 // on the listed path) writes the total and the overflow flag.
 template <typename E>
-__global__ void __launch_bounds__(1024) k4_emit_listed(const E *__restrict__ plane, int64_t nb, int zmax, LevelTable lt,
+__global__ void __launch_bounds__(1024, 1) k4_emit_listed(const E *__restrict__ plane, int64_t nb, int zmax, LevelTable lt,
                                                        int64_t n_units, const int32_t *__restrict__ unit_count,
                                                        const uint32_t *__restrict__ unit_mask,
                                                        fdas_peak *__restrict__ out, int max_peaks, uint32_t series,
                                                        int32_t *__restrict__ npeaks, int32_t *__restrict__ status) {
-    __shared__ uint32_t key[PEAK_LIST_CAP], sorted[PEAK_LIST_CAP];
-    __shared__ int32_t offs[PEAK_LIST_CAP];
+    __shared__ uint32_t key[PEAK_LIST_CAP];
+    __shared__ int32_t cnt[PEAK_LIST_CAP];
     __shared__ int32_t warp_tot[33];
     const int t = threadIdx.x, warp = t >> 5;
     const unsigned int *list = unit_list(unit_count);
@@ -822,33 +1093,39 @@ __global__ void __launch_bounds__(1024) k4_emit_listed(const E *__restrict__ pla
     int64_t total = 0;
     bool writer = false;                                 // the block that writes the total
     if (n <= PEAK_LIST_CAP) {                            // grid-uniform
-        if (blockIdx.x != 0) return;
-        writer = true;
-        if (t < n) key[t] = list[4 + t];
-        __syncthreads();
-        if (t < n) {
-            const uint32_t k = key[t];
-            int rank = 0;
-            for (int j = 0; j < n; j++) rank += key[j] < k;
-            sorted[rank] = k;
+        if (blockIdx.x != 0 && (int)blockIdx.x >= n) return;
+        writer = blockIdx.x == 0;
+        for (int k = t; k < n; k += 1024) {
+            key[k] = list[4 + k];
+            cnt[k] = unit_count[key[k]];
         }
         __syncthreads();
-        // at most 1024 units x 512 peaks: 32-bit offsets
-        const int32_t c = t < n ? unit_count[sorted[t]] : 0;
-        int32_t tot;
-        const int32_t ex = block_excl_scan(c, warp_tot, &tot);
-        if (t < n) offs[t] = ex;
-        total = tot;
-        __syncthreads();
-        for (int k = warp; k < n; k += 32)
-            emit_unit<E>(plane, nb, zmax, lt, (int64_t)sorted[k], offs[k], unit_mask, out, max_peaks, series);
+        // at most 4096 units x 512 peaks: 32-bit offsets
+        const int lane = t & 31;
+        for (int k = (int)blockIdx.x + warp * (int)gridDim.x; k < n; k += 32 * (int)gridDim.x) {
+            const uint32_t mine = key[k];
+            int before = 0;
+            for (int j = lane; j < n; j += 32) before += key[j] < mine ? cnt[j] : 0;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+            emit_unit<E>(plane, nb, zmax, lt.anchored != 0, unit_of(lt, mine), (int64_t)mine, before, unit_mask, out, max_peaks,
+                         series);
+        }
+        if (writer && warp == 31) {
+            int all = 0;
+            for (int j = lane; j < n; j += 32) all += cnt[j];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(0xffffffffu, all, o);
+            total = all;
+        }
+        writer = writer && warp == 31;
     } else {
         // this block's units [ub, ue) (whole rounds of 4096) and the count before them
         const int64_t rounds = (n_units + 4095) / 4096;
         const int64_t per = (rounds + gridDim.x - 1) / gridDim.x;
         const int64_t ub = min(n_units, (int64_t)blockIdx.x * per * 4096);
         const int64_t ue = min(n_units, ub + per * 4096);
-        writer = blockIdx.x == gridDim.x - 1;
+        writer = blockIdx.x == gridDim.x - 1 && warp == 0;
         {
             __shared__ unsigned long long pre_tot;       // counts are non-negative
             if (t == 0) pre_tot = 0ull;
@@ -877,15 +1154,16 @@ __global__ void __launch_bounds__(1024) k4_emit_listed(const E *__restrict__ pla
                     const int j = __ffs(busy) - 1;
                     busy &= busy - 1;
                     const int32_t off_j = __shfl_sync(0xffffffffu, mine, j);
-                    emit_unit<E>(plane, nb, zmax, lt, u0 + 4 * (32 * warp + j) + k, total + off_j, unit_mask, out,
-                                 max_peaks, series);
+                    const int64_t u = u0 + 4 * (32 * warp + j) + k;
+                    emit_unit<E>(plane, nb, zmax, lt.anchored != 0, unit_of(lt, u), u, total + off_j, unit_mask, out, max_peaks,
+                                 series);
                 }
             }
             total += tot;
             __syncthreads();                             // warp_tot is reused by the next round
         }
     }
-    if (writer && t == 0) {
+    if (writer && (t & 31) == 0) {
         *npeaks = (int32_t)(total < 0x7fffffff ? total : 0x7fffffff);
         if (total > max_peaks) atomicOr(status, FDAS_DEV_PEAK_OVERFLOW);
     }
@@ -915,14 +1193,21 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
     // both already (list_cleared)
     uint32_t *list_hdr = reinterpret_cast<uint32_t *>(unit_count) - PEAK_LIST_WORDS;
     if (!list_cleared) {
-        cudaError_t e0 = cudaMemsetAsync(list_hdr, 0, 2 * sizeof(uint32_t), st);
+        cudaError_t e0 = cudaMemsetAsync(list_hdr, 0, 3 * sizeof(uint32_t), st);
         if (e0 != cudaSuccess) return e0;
     }
     p.prof.launches += lt.n_levels > 1 ? 3 : 2;
+    // whether some level kernel leaves cells above the threshold to k4_verify
+    const bool verify = lt.n_levels > 1 && (lt.anchored || !IN_PLACE<E>);
     // with the marks, the level search's work list is built by extra blocks of the level-1 pass
     const bool select_list = l2mark != nullptr && lt.n_levels > 1 && !lt.anchored && (sizeof(E) == 4 || FDAS_K4_RAY_BF16);
     uint32_t *work = reinterpret_cast<uint32_t *>(ws + p.ws_k4work);
     unsigned int *wcount = select_list ? list_hdr + 1 : nullptr;
+    // from 4096 entries on the list is put in order (one more launch, 4 us; below, the whole region is
+    // a few MB of plane and any order will do): the level search of N = 2^23, 85 templates takes 132 us
+    // instead of 148 (BF16), 170 instead of 190 (FP32); N = 2^21, BF16, 3500 entries of 4 chunks:
+    // 43 instead of 49
+    uint32_t *keep = select_list && p.k4order_n >= 4096 ? work + p.k4order_n : nullptr;
     p.prof.begin(PROF_PEAKS_LEVEL1, st);
     if (l1flag) {
         const int64_t n1 = (int64_t)p.K * chunks1;
@@ -930,11 +1215,15 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
         const int64_t n_sel = select_list ? p.k4order_n : 0;
         const int64_t sel_blocks = (n_sel + DETECT_WARPS * 32 - 1) / (DETECT_WARPS * 32);
         k4_level1_marked<E><<<(unsigned)(blocks + sel_blocks), DETECT_WARPS * 32, 0, st>>>(
-            plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], n1, l1flag, unit_count, unit_mask, blocks, p.d_k4order, n_sel,
-            lt, (int)chunks2, work);
+            plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], !verify, n1, l1flag, unit_count, unit_mask, blocks, p.d_k4order, n_sel,
+            lt, (int)chunks2, work, keep);
+        if (keep) {
+            k4_compact<<<(unsigned)((p.k4order_n + 255) / 256), 256, 0, st>>>(keep, p.d_k4order, p.k4order_n, work, wcount);
+            p.prof.launches++;
+        }
         p.prof.level1_fused++;
     } else {
-        k4_level1<E><<<level1_grid, DETECT_WARPS * 32, 0, st>>>(plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], (int)chunks1,
+        k4_level1<E><<<level1_grid, DETECT_WARPS * 32, 0, st>>>(plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], (int)chunks1, !verify,
                                                                  unit_count, unit_mask);
     }
     p.prof.end(PROF_PEAKS_LEVEL1, st);
@@ -953,9 +1242,10 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
     } else if (lt.n_levels > 1) {
         p.prof.begin(PROF_PEAKS_LEVELS, st);
         if (sizeof(E) == 4 || FDAS_K4_RAY_BF16) {
-            // BF16 plane: a persistent grid (0.182 ms against 0.238 ms for one block per entry at
-            // N = 2^23, 85 templates); FP32 plane: one block per entry (0.219 ms against 0.322 ms
-            // persistent, its entries carry twice the bytes and the static stride balances worse)
+            // BF16 plane: a persistent grid (whole region, N = 2^23, 85 templates: 0.191 ms, one block
+            // per entry 0.26; entries drawn from a counter 0.22).  FP32 plane: one block per entry
+            // (with the marks' list 0.170 ms, persistent 0.268: its entries carry twice the bytes and
+            // the static stride balances worse; drawn from a counter 0.188)
             int sms = 0;
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p.device >= 0 ? p.device : 0);
             const int64_t blocks = sizeof(E) == 4 ? p.k4order_n
@@ -973,9 +1263,17 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
         }
         p.prof.end(PROF_PEAKS_LEVELS, st);
     }
-    // one block per SM: block 0 serves the usual (listed) case, all of them the overflowing one
     int sms_out = 152;
     cudaDeviceGetAttribute(&sms_out, cudaDevAttrMultiProcessorCount, p.device >= 0 ? p.device : 0);
+    if (verify) {
+        const int64_t group = lt.anchored ? DETECT_WARPS : DETECT_WARPS * CPW;
+        const int64_t n_order = (int64_t)lt.lev[1].rows * ((lt.lev[1].chunks + group - 1) / group);
+        const uint32_t *order = !lt.anchored ? p.d_k4order : p.k4order_a_n == n_order ? p.d_k4order_a : nullptr;
+        k4_verify<E><<<(unsigned)std::max(1, 4 * sms_out), VERIFY_WARPS * 32, 0, st>>>(plane, p.nb, p.cfg.zmax, p.K, lt, order,
+                                                                                      n_order, unit_count, unit_mask);
+        p.prof.launches++;
+    }
+    // one block per SM: a listed unit per block and warp in the usual case, a range of all units each else
     k4_emit_listed<E><<<(unsigned)std::max(1, sms_out), 1024, 0, st>>>(
         plane, p.nb, p.cfg.zmax, lt, n_units, unit_count, unit_mask, peaks, p.cfg.max_peaks, series, npeaks, p.d_status);
     p.prof.end(FDAS_STAGE_PEAKS, st);
