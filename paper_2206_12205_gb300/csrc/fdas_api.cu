@@ -58,23 +58,23 @@ __global__ void wait_check(int64_t max_cycles, int32_t *status) {
 }
 
 cudaError_t launch_plane_any(const Plan &p, const float2 *x, const float *scale, char *ws, void *d_plane,
-                             cudaStream_t st, uint8_t *l1flag) {
+                             cudaStream_t st, uint8_t *l1flag, bool early) {
     switch (p.cfg.precision) {
-        case FDAS_BF16: return launch_plane_bf16(p, x, scale, ws, static_cast<__nv_bfloat16 *>(d_plane), st, l1flag);
+        case FDAS_BF16: return launch_plane_bf16(p, x, scale, ws, static_cast<__nv_bfloat16 *>(d_plane), st, l1flag, early);
         case FDAS_BF16_SPLIT: return launch_plane_split(p, x, scale, ws, static_cast<float *>(d_plane), st);
-        case FDAS_FP16_SCALED: return launch_plane_f16(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag);
+        case FDAS_FP16_SCALED: return launch_plane_f16(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag, early);
         case FDAS_BF16_DIRECT:
             return launch_plane_direct(p, x, scale, static_cast<__nv_bfloat16 *>(d_plane), st, l1flag);
         case FDAS_FP8_DIRECT: return launch_plane_direct_f8(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag);
-        default: return launch_plane_fp32(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag);
+        default: return launch_plane_fp32(p, x, scale, ws, static_cast<float *>(d_plane), st, l1flag, early);
     }
 }
 }  // namespace fdas
 
 namespace {
 cudaError_t launch_plane_any(Plan *p, const float2 *x, const float *scale, char *ws, void *d_plane, cudaStream_t st,
-                             uint8_t *l1flag = nullptr) {
-    return fdas::launch_plane_any(*p, x, scale, ws, d_plane, st, l1flag);
+                             uint8_t *l1flag = nullptr, bool early = false) {
+    return fdas::launch_plane_any(*p, x, scale, ws, d_plane, st, l1flag, early);
 }
 }  // namespace
 
@@ -311,7 +311,8 @@ fdas_status fdas_search(fdas_plan_t plan, const float *d_series, void *d_workspa
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *ws = static_cast<char *>(d_workspace);
     p->prof.calls++;
-    cudaError_t e = fdas::launch_spectrum(*p, d_series, ws, st);
+    const bool early = p->nb <= fdas::launch_early_bins(p->device);
+    cudaError_t e = fdas::launch_spectrum(*p, d_series, ws, st, early);
     float2 *x = reinterpret_cast<float2 *>(ws + p->ws_x);
     const float *scale = reinterpret_cast<const float *>(ws + p->ws_scale + 8);
     if (e == cudaSuccess && p->cfg.norm_block) {      // normalised in place, no global scale
@@ -320,9 +321,9 @@ fdas_status fdas_search(fdas_plan_t plan, const float *d_series, void *d_workspa
     }
     // the tensor-core plane kernels mark the level-1 units as they store the plane
     uint8_t *l1flag = fdas::level1_fusable(*p) ? reinterpret_cast<uint8_t *>(ws + p->ws_l1flag) : nullptr;
-    if (e == cudaSuccess) e = launch_plane_any(p, x, scale, ws, d_plane, st, l1flag);
+    if (e == cudaSuccess) e = launch_plane_any(p, x, scale, ws, d_plane, st, l1flag, early);
     if (e == cudaSuccess)
-        e = fdas::launch_peaks(*p, d_plane, plane_is_bf16(p), ws, d_peaks, d_npeaks, 0u, st, l1flag, true);
+        e = fdas::launch_peaks(*p, d_plane, plane_is_bf16(p), ws, d_peaks, d_npeaks, 0u, st, l1flag, true, early);
     return record(p, e);
 }
 

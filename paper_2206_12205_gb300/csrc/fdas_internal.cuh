@@ -128,21 +128,56 @@ LevelTable make_levels(const Plan &p);
 // n-point Gauss-Legendre nodes xs and weights ws on [-1, 1] (host, FP64).
 void gauss_legendre(int n, double *xs, double *ws);
 
+// Programmatic dependent launch.  A kernel launched with launch_after(early = true) may become
+// resident, and do what does not depend on the kernels before it (tables, barriers, TMEM), while the
+// last of those finishes; grid_wait() then holds it until that one has completed and its writes are
+// visible.  Its blocks pass grid_wait() before they touch memory that other kernels write or read, and
+// call grid_release() (which lets the next kernel's blocks in, once every block has called it or
+// exited) only after that: so when a kernel starts, all but the last kernel before it have completed,
+// and only what that last one writes has to be read with plain loads instead of the read-only path.
+//   early: a search by itself of at most launch_early_bins() bins, whose kernels are short enough that
+// the gaps between them count (N = 2^16, FP32, 64 taps: 50.5 -> 35 us; N = 2^18, BF16: 72 -> 62 us; BF16
+// N = 2^19: 82 -> 75 us).  On larger ones a plane kernel that waits beside the segment FFTs' last waves
+// costs more than the gap (BF16, N = 2^20: 116 -> 123 us; N = 2^23: 588 -> 608 us), and in batches blocks that wait keep the
+// other lanes' out (12 series of 2^21, 3 lanes: 3.32 -> 3.52 ms); these launch plainly, which makes
+// both calls no-ops.
+inline int64_t launch_early_bins(int device) {
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device >= 0 ? device : 0);
+    return (int64_t)sms * 2048;                      // N = 2^19 on 152 SMs
+}
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_after(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- launchers (each returns cudaGetLastError() of its launches) ----
 cudaError_t launch_make_templates(Plan &p, cudaStream_t st);
-cudaError_t launch_spectrum(const Plan &p, const float *d_series, char *ws, cudaStream_t st);
+cudaError_t launch_spectrum(const Plan &p, const float *d_series, char *ws, cudaStream_t st, bool early = false);
 cudaError_t launch_local_norm(const Plan &p, const float2 *d_x, float2 *d_out, cudaStream_t st);
 cudaError_t launch_apply_scale(const Plan &p, const char *ws, float *d_xhat, double *d_sigma2,
                                cudaStream_t st);
 cudaError_t launch_plane_fp32(const Plan &p, const float2 *d_x, const float *d_scale, char *ws,
-                              float *d_plane, cudaStream_t st, uint8_t *l1flag = nullptr);
+                              float *d_plane, cudaStream_t st, uint8_t *l1flag = nullptr, bool early = false);
 // The same kernels with the segment spectra (n_seg * S complex64) at d_yhat instead of the workspace.
 cudaError_t launch_plane_fp32_scratch(const Plan &p, const float2 *d_x, const float *d_scale, float2 *d_yhat,
                                       float *d_plane, cudaStream_t st);
-// l1flag (optional, K x Nb/512 bytes): the plane kernel zeroes it and marks every 512-bin unit of
+// l1flag (optional, K x Nb/512 bytes): the call zeroes it and marks every 512-bin unit of
 // a row holding a stored value above the level-1 threshold (the level-1 pass then reads only those).
 cudaError_t launch_plane_bf16(const Plan &p, const float2 *d_x, const float *d_scale, char *ws,
-                              __nv_bfloat16 *d_plane, cudaStream_t st, uint8_t *l1flag = nullptr);
+                              __nv_bfloat16 *d_plane, cudaStream_t st, uint8_t *l1flag = nullptr, bool early = false);
 cudaError_t launch_prepare_bf16(Plan &p, cudaStream_t st);
 // FP32 segment spectra for 4096-bin segments (the split-BF16 path's input).
 cudaError_t launch_segments_fp32(const Plan &p, const float2 *d_x, const float *d_scale, float2 *d_yhat,
@@ -156,7 +191,7 @@ cudaError_t launch_plane_direct_f8(const Plan &p, const float2 *d_x, const float
 cudaError_t launch_plane_direct(const Plan &p, const float2 *d_x, const float *d_scale, __nv_bfloat16 *d_plane,
                                 cudaStream_t st, uint8_t *l1flag = nullptr);
 cudaError_t launch_plane_f16(const Plan &p, const float2 *d_x, const float *d_scale, char *ws, float *d_plane,
-                             cudaStream_t st, uint8_t *l1flag = nullptr);
+                             cudaStream_t st, uint8_t *l1flag = nullptr, bool early = false);
 // Whether the plan's plane kernel marks the level-1 units (every precision's plane kernel).
 bool level1_fusable(const Plan &p);
 // The threshold of the plane kernels' unit marks: a 512-bin unit is marked when it holds a stored
@@ -169,7 +204,7 @@ inline float mark_threshold(const Plan &p) {
 }
 // The plane of the plan's precision from a spectrum (x: Nb complex; scale: device factor or NULL).
 cudaError_t launch_plane_any(const Plan &p, const float2 *x, const float *scale, char *ws, void *d_plane,
-                             cudaStream_t st, uint8_t *l1flag = nullptr);
+                             cudaStream_t st, uint8_t *l1flag = nullptr, bool early = false);
 // l1flag: the unit marks of the plane kernel that wrote d_plane (level 1 then visits only the
 // marked units), or NULL for the full level-1 pass over the plane.
 // The ray order of level 2's blocks (host; false if the region does not fit the 16-bit fields),
@@ -181,7 +216,7 @@ cudaError_t upload_levels_order(Plan &p);
 // earlier on the stream (launch_spectrum does); else the peak search clears them itself.
 cudaError_t launch_peaks(const Plan &p, const void *d_plane, bool bf16, char *ws,
                          fdas_peak *d_peaks, int32_t *d_npeaks, uint32_t series, cudaStream_t st,
-                         const uint8_t *l1flag = nullptr, bool list_cleared = false);
+                         const uint8_t *l1flag = nullptr, bool list_cleared = false, bool early = false);
 cudaError_t launch_band_max(const Plan &p, const void *d_plane, bool bf16, const int64_t *d_lo, const int64_t *d_hi,
                             int n_bands, int64_t max_width, unsigned long long *d_slot, float *d_value,
                             int64_t *d_r, int32_t *d_zi, cudaStream_t st);

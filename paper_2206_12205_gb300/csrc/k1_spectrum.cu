@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(k1_groups_a(M1) * (M1 / 32), FDAS_K1A_MIN_BLOC
     extern __shared__ float2 sm[];        // C1 * E entries
     __shared__ float2 wi[C1][33];         // W_N^{2 n2 T i} of each column (rows padded: the groups of a
                                           // warp read one entry each, on different banks)
+    grid_release();
     const int g = threadIdx.x % C1, t = threadIdx.x / C1;
     const int n2 = blockIdx.x * C1 + g;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -130,12 +131,12 @@ __device__ __forceinline__ void k1_sum_and_finalize(float acc, double *red, doub
 // Groups 0 .. C2-1 take rows a = p C2 + g; groups C2 .. 2 C2 - 1 their partners M1 - a (row 0,
 // its own partner, lends its partner slot to row M1/2, the other self-partnered row).
 template <int M2>
-__global__ void __launch_bounds__(2 * k1_groups_b(M2) * (M2 / 32), FDAS_K1B_MIN_BLOCKS) k1_pass_b(const float2 *__restrict__ B,
+__global__ void __launch_bounds__(2 * k1_groups_b(M2) * (M2 / 32), FDAS_K1B_MIN_BLOCKS) k1_pass_b(const float2 *B,
                                                                          const float2 *__restrict__ tw,
                                                                          const float2 *__restrict__ lo,
                                                                          const float2 *__restrict__ hi,
-                                                                         float2 *__restrict__ X,
-                                                                         double *__restrict__ partial, int M1,
+                                                                         float2 *X,
+                                                                         double *partial, int M1,
                                                                          unsigned int *__restrict__ ticket, int64_t nb,
                                                                          double sigma2_fixed, double *__restrict__ sigma2_out,
                                                                          float *__restrict__ scale_out) {
@@ -149,9 +150,11 @@ __global__ void __launch_bounds__(2 * k1_groups_b(M2) * (M2 / 32), FDAS_K1B_MIN_
     float2 *sm = smb + g * E;
     __shared__ float2 w64[32];            // W_N^{M1 T i} = W_64^i
     for (int i = threadIdx.x; i < 32; i += G * T) w64[i] = twN(lo, hi, (int64_t)M1 * T * i);
+    grid_wait();
+    grid_release();
     float2 v[32];
 #pragma unroll
-    for (int i = 0; i < 32; i++) v[i] = __ldg(B + (int64_t)row * M2 + t + i * T);
+    for (int i = 0; i < 32; i++) v[i] = B[(int64_t)row * M2 + t + i * T];
     block_fft<M2>(v, sm, tw, t);
     // the last FFT stage works in registers and the previous exchange ended with a barrier
 #pragma unroll
@@ -251,20 +254,19 @@ cudaError_t run_pass_a(const Plan &p, const float2 *z, float2 *B, unsigned int *
 
 template <int M2>
 cudaError_t run_pass_b(const Plan &p, const float2 *B, float2 *X, double *partial, unsigned int *ticket,
-                       double *sigma2, float *scale, cudaStream_t st) {
+                       double *sigma2, float *scale, cudaStream_t st, bool early) {
     constexpr int C2 = k1_groups_b(M2);
     const size_t smem = 2 * C2 * sizeof(float2) * k1_region(M2, 2 * C2);
     auto kern = k1_pass_b<M2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<p.M1 / (2 * C2), 2 * C2 * (M2 / 32), smem, st>>>(B, p.d_tw, p.d_twn_lo, p.d_twn_hi, X, partial, p.M1,
-                                                              ticket, p.nb, p.cfg.sigma2, sigma2, scale);
-    return cudaGetLastError();
+    return launch_after(early, kern, p.M1 / (2 * C2), 2 * C2 * (M2 / 32), smem, st, B, p.d_tw, p.d_twn_lo, p.d_twn_hi, X, partial, p.M1,
+                        ticket, p.nb, p.cfg.sigma2, sigma2, scale);
 }
 
 }  // namespace
 
-cudaError_t launch_spectrum(const Plan &p, const float *d_series, char *ws, cudaStream_t st) {
+cudaError_t launch_spectrum(const Plan &p, const float *d_series, char *ws, cudaStream_t st, bool early) {
     const float2 *z = reinterpret_cast<const float2 *>(d_series);
     float2 *B = reinterpret_cast<float2 *>(ws + p.ws_tmp);
     float2 *X = reinterpret_cast<float2 *>(ws + p.ws_x);
@@ -290,15 +292,15 @@ cudaError_t launch_spectrum(const Plan &p, const float *d_series, char *ws, cuda
     if (e != cudaSuccess) return e;
     e = cudaErrorInvalidValue;
     switch (p.M2) {
-        case 32: e = run_pass_b<32>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 64: e = run_pass_b<64>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 128: e = run_pass_b<128>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 256: e = run_pass_b<256>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 512: e = run_pass_b<512>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 1024: e = run_pass_b<1024>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 2048: e = run_pass_b<2048>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 4096: e = run_pass_b<4096>(p, B, X, partial, ticket, sigma2, scale, st); break;
-        case 8192: e = run_pass_b<8192>(p, B, X, partial, ticket, sigma2, scale, st); break;
+        case 32: e = run_pass_b<32>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 64: e = run_pass_b<64>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 128: e = run_pass_b<128>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 256: e = run_pass_b<256>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 512: e = run_pass_b<512>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 1024: e = run_pass_b<1024>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 2048: e = run_pass_b<2048>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 4096: e = run_pass_b<4096>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
+        case 8192: e = run_pass_b<8192>(p, B, X, partial, ticket, sigma2, scale, st, early); break;
     }
     if (e != cudaSuccess) return e;
     p.prof.end(FDAS_STAGE_SPECTRUM, st);

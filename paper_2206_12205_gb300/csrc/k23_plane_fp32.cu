@@ -33,16 +33,20 @@ constexpr size_t f16_smem(bool db) {
 // K2: the segment spectra.  Each CTA transforms segments j = blockIdx.x, blockIdx.x + gridDim.x, ...
 // (the shared twiddle table is filled once per CTA).
 template <int S>
-__global__ void __launch_bounds__(S / 16) k2_segments(const float2 *__restrict__ X, const float *__restrict__ scale_ptr,
-                                                      const float2 *__restrict__ tw, float2 *__restrict__ Y,
-                                                      int64_t n_seg, int64_t nb, int L, int half_m) {
+__global__ void __launch_bounds__(S / 16) k2_segments(const float2 *X, const float *scale_ptr, const float2 *__restrict__ tw,
+                                                      float2 *__restrict__ Y, int64_t n_seg, int64_t nb, int L, int half_m,
+                                                      uint4 *zero16, int64_t n_zero16) {
     constexpr int T = S / 16;
     extern __shared__ float2 sm[];
     float2 *tws = sm;
     float2 *xs = sm + f16_tw_entries(S);
     const int t = threadIdx.x;
     f16_load_twiddles<S>(tws, tw, t);
-    const float scale = scale_ptr ? __ldg(scale_ptr) : 1.0f;
+    grid_wait();
+    grid_release();
+    // the plane kernel's unit marks (whole 16-byte words), which saves it a separate clearing
+    for (int64_t w = (int64_t)blockIdx.x * T + t; w < n_zero16; w += (int64_t)gridDim.x * T) zero16[w] = make_uint4(0u, 0u, 0u, 0u);
+    const float scale = scale_ptr ? *scale_ptr : 1.0f;
     for (int64_t j = blockIdx.x; j < n_seg; j += gridDim.x) {
         const int64_t base = j * L - half_m;
         float2 v[16];
@@ -50,7 +54,7 @@ __global__ void __launch_bounds__(S / 16) k2_segments(const float2 *__restrict__
         for (int i = 0; i < 16; i++) {
             const int64_t k = base + t + i * T;
             float2 x = make_float2(0.f, 0.f);
-            if (k >= 0 && k < nb) x = __ldg(X + k);
+            if (k >= 0 && k < nb) x = X[k];
             v[i] = make_float2(x.x * scale, x.y * scale);
         }
         block_fft16<S, false>(v, xs, xs, tws, t);
@@ -64,7 +68,7 @@ __global__ void __launch_bounds__(S / 16) k2_segments(const float2 *__restrict__
 // PRE: the segment spectrum stays in registers and the next template's spectrum is loaded while
 // the current transform runs (its L2 latency is then hidden behind the FFT).
 template <int S, bool DB, int MINB, bool PRE>
-__global__ void __launch_bounds__(S / 16, MINB) k3_plane_fp32(const float2 *__restrict__ Y, const float2 *__restrict__ G,
+__global__ void __launch_bounds__(S / 16, MINB) k3_plane_fp32(const float2 *Y, const float2 *__restrict__ G,
                                                              const float2 *__restrict__ tw, float *__restrict__ plane,
                                                              int K, int groups, int64_t nb, int L,
                                                              uint8_t *__restrict__ l1flag, int64_t chunks1, float thr1) {
@@ -75,6 +79,8 @@ __global__ void __launch_bounds__(S / 16, MINB) k3_plane_fp32(const float2 *__re
     float2 *xb = DB ? xa + f16_xchg_entries(S) : xa;
     const int t = threadIdx.x;
     f16_load_twiddles<S>(tws, tw, t);
+    grid_wait();
+    grid_release();
     // segment-major block order: consecutive blocks write consecutive stretches of the same rows
     // (with the groups of a segment adjacent instead, its spectrum came from DRAM once, 40 MB
     // instead of 232 MB read at N = 2^23, but the kernel took 0.943 ms instead of 0.926 ms)
@@ -92,7 +98,7 @@ __global__ void __launch_bounds__(S / 16, MINB) k3_plane_fp32(const float2 *__re
             const float2 *Gz = G + (int64_t)z0 * S;
 #pragma unroll
             for (int i = 0; i < 16; i++) {
-                y[i] = __ldg(Yj + t + i * T);
+                y[i] = Yj[t + i * T];
                 g[i] = __ldg(Gz + t + i * T);
             }
         }
@@ -112,7 +118,7 @@ __global__ void __launch_bounds__(S / 16, MINB) k3_plane_fp32(const float2 *__re
 #pragma unroll
             for (int i = 0; i < 16; i++) {
                 const int k = t + i * T;
-                v[i] = cmul_conj_a(__ldg(Yj + k), __ldg(Gz + k));
+                v[i] = cmul_conj_a(Yj[k], __ldg(Gz + k));
             }
         }
         block_fft16<S, DB>(v, xa, xb, tws, t);
@@ -144,21 +150,24 @@ int sm_count(const Plan &p) {
 }
 
 template <int S>
-cudaError_t run_segments(const Plan &p, const float2 *d_x, const float *d_scale, float2 *Y, cudaStream_t st) {
+cudaError_t run_segments(const Plan &p, const float2 *d_x, const float *d_scale, float2 *Y, cudaStream_t st, uint8_t *l1flag, bool early) {
     const size_t smem = f16_smem<S>(false);
     cudaError_t e = cudaFuncSetAttribute(k2_segments<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // enough CTAs to fill every SM a few times; each fills its twiddle table once
     const int64_t grid = std::min<int64_t>(p.n_seg, (int64_t)sm_count(p) * std::max(1, 4096 / S) * 2);
     p.prof.begin(FDAS_STAGE_SEGMENTS, st);
-    k2_segments<S><<<(unsigned)grid, S / 16, smem, st>>>(d_x, d_scale, p.d_tw, Y, p.n_seg, p.nb, p.L, p.m / 2);
+    // the unit marks' workspace slot is 256-byte aligned and padded: whole 16-byte words cover it
+    const int64_t n_zero16 = l1flag ? ((int64_t)p.K * (p.nb / PEAK_CHUNK) + 15) / 16 : 0;
+    e = launch_after(early, k2_segments<S>, (unsigned)grid, S / 16, smem, st, d_x, d_scale, p.d_tw, Y, p.n_seg, p.nb, p.L, p.m / 2,
+                     reinterpret_cast<uint4 *>(l1flag), n_zero16);
     p.prof.end(FDAS_STAGE_SEGMENTS, st);
     p.prof.launches += 1;
-    return cudaGetLastError();
+    return e;
 }
 
 template <int S, bool DB, int MINB, bool PRE>
-cudaError_t run_correlate(const Plan &p, const float2 *Y, float *plane, cudaStream_t st, uint8_t *l1flag) {
+cudaError_t run_correlate(const Plan &p, const float2 *Y, float *plane, cudaStream_t st, uint8_t *l1flag, bool early) {
     const size_t smem = f16_smem<S>(DB);
     cudaError_t e = cudaFuncSetAttribute(k3_plane_fp32<S, DB, MINB, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
@@ -168,16 +177,12 @@ cudaError_t run_correlate(const Plan &p, const float2 *Y, float *plane, cudaStre
     if (p.tune_zb > 0) zb = std::min(p.tune_zb, p.K);
     const int groups = (p.K + zb - 1) / zb;
     const int64_t grid = p.n_seg * groups;
-    if (l1flag) {
-        e = cudaMemsetAsync(l1flag, 0, (size_t)p.K * (size_t)(p.nb / PEAK_CHUNK), st);
-        if (e != cudaSuccess) return e;
-    }
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    k3_plane_fp32<S, DB, MINB, PRE><<<(unsigned)grid, S / 16, smem, st>>>(Y, p.d_G, p.d_tw, plane, p.K, groups, p.nb,
-                                                                        p.L, l1flag, p.nb / PEAK_CHUNK, mark_threshold(p));
+    e = launch_after(early, k3_plane_fp32<S, DB, MINB, PRE>, (unsigned)grid, S / 16, smem, st, Y, p.d_G, p.d_tw, plane, p.K, groups, p.nb,
+                     p.L, l1flag, p.nb / PEAK_CHUNK, mark_threshold(p));
     p.prof.end(FDAS_STAGE_CORRELATE, st);
     p.prof.launches += 1;
-    return cudaGetLastError();
+    return e;
 }
 
 // Launch shapes, measured at N = 2^23, 85 templates, 256 taps (correlation kernel, ms):
@@ -190,13 +195,13 @@ cudaError_t run_correlate(const Plan &p, const float2 *Y, float *plane, cudaStre
 // measured faster at any S.
 template <int S>
 cudaError_t run_plane(const Plan &p, const float2 *d_x, const float *d_scale, float2 *Y, float *plane,
-                      cudaStream_t st, uint8_t *l1flag) {
-    cudaError_t e = run_segments<S>(p, d_x, d_scale, Y, st);
+                      cudaStream_t st, uint8_t *l1flag, bool early) {
+    cudaError_t e = run_segments<S>(p, d_x, d_scale, Y, st, l1flag, early);
     if (e != cudaSuccess) return e;
-    if constexpr (S == 8192) return run_correlate<S, false, 1, false>(p, Y, plane, st, l1flag);
-    else if constexpr (S == 4096) return run_correlate<S, true, 2, false>(p, Y, plane, st, l1flag);
-    else if constexpr (S == 2048) return run_correlate<S, false, 3, true>(p, Y, plane, st, l1flag);
-    else return run_correlate<S, true, 8, false>(p, Y, plane, st, l1flag);
+    if constexpr (S == 8192) return run_correlate<S, false, 1, false>(p, Y, plane, st, l1flag, early);
+    else if constexpr (S == 4096) return run_correlate<S, true, 2, false>(p, Y, plane, st, l1flag, early);
+    else if constexpr (S == 2048) return run_correlate<S, false, 3, true>(p, Y, plane, st, l1flag, early);
+    else return run_correlate<S, true, 8, false>(p, Y, plane, st, l1flag, early);
 }
 
 }  // namespace
@@ -204,13 +209,13 @@ cudaError_t run_plane(const Plan &p, const float2 *d_x, const float *d_scale, fl
 static_assert(PEAK_CHUNK == 512, "the level-1 marks index units as bin >> 9");
 
 cudaError_t launch_plane_fp32(const Plan &p, const float2 *d_x, const float *d_scale, char *ws, float *d_plane,
-                              cudaStream_t st, uint8_t *l1flag) {
+                              cudaStream_t st, uint8_t *l1flag, bool early) {
     float2 *Y = reinterpret_cast<float2 *>(ws + p.ws_y);
     switch (p.S) {
-        case 1024: return run_plane<1024>(p, d_x, d_scale, Y, d_plane, st, l1flag);
-        case 2048: return run_plane<2048>(p, d_x, d_scale, Y, d_plane, st, l1flag);
-        case 4096: return run_plane<4096>(p, d_x, d_scale, Y, d_plane, st, l1flag);
-        case 8192: return run_plane<8192>(p, d_x, d_scale, Y, d_plane, st, l1flag);
+        case 1024: return run_plane<1024>(p, d_x, d_scale, Y, d_plane, st, l1flag, early);
+        case 2048: return run_plane<2048>(p, d_x, d_scale, Y, d_plane, st, l1flag, early);
+        case 4096: return run_plane<4096>(p, d_x, d_scale, Y, d_plane, st, l1flag, early);
+        case 8192: return run_plane<8192>(p, d_x, d_scale, Y, d_plane, st, l1flag, early);
     }
     return cudaErrorInvalidValue;
 }
@@ -218,16 +223,16 @@ cudaError_t launch_plane_fp32(const Plan &p, const float2 *d_x, const float *d_s
 cudaError_t launch_segments_fp32(const Plan &p, const float2 *d_x, const float *d_scale, float2 *d_yhat,
                                  cudaStream_t st) {
     if (p.S != 4096) return cudaErrorInvalidValue;
-    return run_segments<4096>(p, d_x, d_scale, d_yhat, st);
+    return run_segments<4096>(p, d_x, d_scale, d_yhat, st, nullptr, false);
 }
 
 cudaError_t launch_plane_fp32_scratch(const Plan &p, const float2 *d_x, const float *d_scale, float2 *d_yhat,
                                       float *d_plane, cudaStream_t st) {
     switch (p.S) {
-        case 1024: return run_plane<1024>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr);
-        case 2048: return run_plane<2048>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr);
-        case 4096: return run_plane<4096>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr);
-        case 8192: return run_plane<8192>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr);
+        case 1024: return run_plane<1024>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr, false);
+        case 2048: return run_plane<2048>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr, false);
+        case 4096: return run_plane<4096>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr, false);
+        case 8192: return run_plane<8192>(p, d_x, d_scale, d_yhat, d_plane, st, nullptr, false);
     }
     return cudaErrorInvalidValue;
 }

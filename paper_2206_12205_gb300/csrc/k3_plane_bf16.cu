@@ -81,8 +81,7 @@ struct OpsF16 {
 // Segment FFTs (FP32 CUDA-core block FFT), stored as BF16 pairs in the stage-1 order.
 // It also clears the plane kernel's unit marks (zero16: n_zero16 16-byte words, or none), which
 // saves the plane kernel a separate clearing launch.
-__global__ void __launch_bounds__(TC_S_BF16 / 32) k2_segments_bf16(const float2 *__restrict__ X,
-                                                                   const float *__restrict__ scale_ptr,
+__global__ void __launch_bounds__(TC_S_BF16 / 32) k2_segments_bf16(const float2 *X, const float *scale_ptr,
                                                                    const float2 *__restrict__ tw,
                                                                    uint4 *__restrict__ Y, int64_t nb, int L,
                                                                    int half_m, uint4 *__restrict__ zero16,
@@ -91,15 +90,17 @@ __global__ void __launch_bounds__(TC_S_BF16 / 32) k2_segments_bf16(const float2 
     extern __shared__ float2 sm[];
     const int t = threadIdx.x;
     const int64_t j = blockIdx.x;
+    grid_wait();
+    grid_release();
     for (int64_t w = j * T + t; w < n_zero16; w += (int64_t)gridDim.x * T) zero16[w] = make_uint4(0u, 0u, 0u, 0u);
-    const float scale = scale_ptr ? __ldg(scale_ptr) : 1.0f;
+    const float scale = scale_ptr ? *scale_ptr : 1.0f;
     const int64_t base = j * L - half_m;
     float2 v[32];
 #pragma unroll
     for (int i = 0; i < 32; i++) {
         const int64_t k = base + t + i * T;
         float2 x = make_float2(0.f, 0.f);
-        if (k >= 0 && k < nb) x = __ldg(X + k);
+        if (k >= 0 && k < nb) x = X[k];
         v[i] = make_float2(x.x * scale, x.y * scale);
     }
     block_fft<S>(v, sm, tw, t);
@@ -115,24 +116,27 @@ __global__ void __launch_bounds__(TC_S_BF16 / 32) k2_segments_bf16(const float2 
 // Segment FFTs for the FP16 stages: the segment's largest component |re| or |im| is brought into
 // [0.5, 1) by a power of two s_j (exact), the values stored as FP16 pairs in the stage-1 order,
 // and the plane's factor 1 / (s_j gscale)^2 (gscale: the template bank's scale) kept per segment.
-__global__ void __launch_bounds__(TC_S_BF16 / 32) k2_segments_f16(const float2 *__restrict__ X,
-                                                                  const float *__restrict__ scale_ptr,
+__global__ void __launch_bounds__(TC_S_BF16 / 32) k2_segments_f16(const float2 *X, const float *scale_ptr,
                                                                   const float2 *__restrict__ tw,
                                                                   uint4 *__restrict__ Y, float *__restrict__ unscale,
-                                                                  float gscale, int64_t nb, int L, int half_m) {
+                                                                  float gscale, int64_t nb, int L, int half_m,
+                                                                  uint4 *__restrict__ zero16, int64_t n_zero16) {
     constexpr int S = TC_S_BF16, T = S / 32;
     extern __shared__ float2 sm[];
     __shared__ float wmax[T / 32];
     const int t = threadIdx.x;
     const int64_t j = blockIdx.x;
-    const float scale = scale_ptr ? __ldg(scale_ptr) : 1.0f;
+    grid_wait();
+    grid_release();
+    for (int64_t w = j * T + t; w < n_zero16; w += (int64_t)gridDim.x * T) zero16[w] = make_uint4(0u, 0u, 0u, 0u);
+    const float scale = scale_ptr ? *scale_ptr : 1.0f;
     const int64_t base = j * L - half_m;
     float2 v[32];
 #pragma unroll
     for (int i = 0; i < 32; i++) {
         const int64_t k = base + t + i * T;
         float2 x = make_float2(0.f, 0.f);
-        if (k >= 0 && k < nb) x = __ldg(X + k);
+        if (k >= 0 && k < nb) x = X[k];
         v[i] = make_float2(x.x * scale, x.y * scale);
     }
     block_fft<S>(v, sm, tw, t);
@@ -251,12 +255,12 @@ __device__ __forceinline__ float2 u2f2(uint32_t a, uint32_t b) {
 }
 
 template <class Ops>
-__global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc(const uint4 *__restrict__ Y, const uint4 *__restrict__ G,
+__global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc(const uint4 *Y, const uint4 *__restrict__ G,
                                                              const uint4 *__restrict__ Fimg,
                                                              const float2 *__restrict__ tw,
                                                              typename Ops::Out *__restrict__ plane, int K, int64_t nb,
                                                              int L, int64_t n_items, int n_groups,
-                                                             int64_t items_per_cta, const float *__restrict__ unscale,
+                                                             int64_t items_per_cta, const float *unscale,
                                                              uint8_t *__restrict__ l1flag, int64_t chunks1, float thr1,
                                                              int32_t *__restrict__ status) {
     using V = typename Ops::V;
@@ -297,6 +301,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc(const uint4 *__rest
     tc::fence_before_thread_sync();
     __syncthreads();
     tc::fence_after_thread_sync();
+    grid_wait();
+    grid_release();
 
     const uint32_t tbase = *tslot;
     const int64_t it0 = (int64_t)blockIdx.x * items_per_cta;
@@ -387,7 +393,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc(const uint4 *__rest
             uint4 yv[8];
             const uint4 *Yj = Yb + j * (TC_S_BF16 / 4);
 #pragma unroll
-            for (int c = 0; c < 8; c++) yv[c] = __ldg(Yj + c * TC_R);
+            for (int c = 0; c < 8; c++) yv[c] = Yj[c * TC_R];
             if (k >= 2 && !ws_wait(&bars->a1_free[sl], (uint32_t)(((k - 2) >> 1) & 1), abort_flag)) break;
             tc::fence_after_thread_sync();
             // conj(y) g: Re = yr gr + yi gi, Im = yr gi - yi gr, two n1 per packed pair; written in
@@ -487,7 +493,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc(const uint4 *__rest
             tc::fence_after_thread_sync();
             const int z = grp * TC_G + zl;
             const int64_t r0 = j * L;
-            const float us = unscale ? __ldg(unscale + j) : 1.0f;
+            const float us = unscale ? unscale[j] : 1.0f;
             if (++j == n_seg) {                         // the next item
                 j = 0;
                 grp++;
@@ -606,7 +612,7 @@ struct SpBars {
     uint64_t a1_full[2], a1_free[2], d1_full[3], b2_full, a2_free, d2_full[3], d_free[3], drain[2];
 };
 
-__global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 *__restrict__ Y,
+__global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 *Y,
                                                                    const float2 *__restrict__ G,
                                                                    const uint4 *__restrict__ Fimg,
                                                                    const float2 *__restrict__ tw,
@@ -649,6 +655,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 
     tc::fence_before_thread_sync();
     __syncthreads();
     tc::fence_after_thread_sync();
+    grid_wait();
+    grid_release();
 
     const uint32_t tbase = *tslot;
     const int64_t it0 = (int64_t)blockIdx.x * items_per_cta;
@@ -741,7 +749,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 
             const float2 *Gp = G + (int64_t)(z < K ? z : 0) * TC_S_BF16 + (32 * hp + 8 * i) * TC_R + n2;
 #pragma unroll
             for (int e = 0; e < 8; e++) {
-                y[e] = __ldg(Yp + e * TC_R);
+                y[e] = Yp[e * TC_R];
                 g[e] = __ldg(Gp + e * TC_R);
             }
         };
@@ -982,14 +990,8 @@ bool level1_fusable(const Plan &p) {
            p.cfg.precision == FDAS_BF16_DIRECT || p.cfg.precision == FDAS_FP8_DIRECT;
 }
 
-// Clear the level-1 unit marks before the plane kernel sets them.
-static cudaError_t clear_marks(const Plan &p, uint8_t *l1flag, cudaStream_t st) {
-    if (!l1flag) return cudaSuccess;
-    return cudaMemsetAsync(l1flag, 0, (size_t)p.K * (size_t)(p.nb / PEAK_CHUNK), st);
-}
-
 cudaError_t launch_plane_bf16(const Plan &p, const float2 *d_x, const float *d_scale, char *ws,
-                              __nv_bfloat16 *d_plane, cudaStream_t st, uint8_t *l1flag) {
+                              __nv_bfloat16 *d_plane, cudaStream_t st, uint8_t *l1flag, bool early) {
     if (p.S != TC_S_BF16) return cudaErrorInvalidValue;
     uint4 *Y = reinterpret_cast<uint4 *>(ws + p.ws_y);
     const size_t smem2 = sizeof(float2) * fft_smem_entries(TC_S_BF16);
@@ -1001,10 +1003,9 @@ cudaError_t launch_plane_bf16(const Plan &p, const float2 *d_x, const float *d_s
     // and padded to 256 bytes, so whole 16-byte words cover it
     const int64_t n_zero16 = l1flag ? ((int64_t)p.K * (p.nb / PEAK_CHUNK) + 15) / 16 : 0;
     p.prof.begin(FDAS_STAGE_SEGMENTS, st);
-    k2_segments_bf16<<<(unsigned)p.n_seg, TC_S_BF16 / 32, smem2, st>>>(d_x, d_scale, p.d_tw, Y, p.nb, p.L, p.m / 2,
-                                                                      reinterpret_cast<uint4 *>(l1flag), n_zero16);
+    e = launch_after(early, k2_segments_bf16, (unsigned)p.n_seg, TC_S_BF16 / 32, smem2, st, d_x, d_scale, p.d_tw, Y, p.nb, p.L, p.m / 2,
+                     reinterpret_cast<uint4 *>(l1flag), n_zero16);
     p.prof.end(FDAS_STAGE_SEGMENTS, st);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int n_groups = (p.K + TC_G - 1) / TC_G;
     const int64_t n_items = p.n_seg * n_groups;
@@ -1014,18 +1015,17 @@ cudaError_t launch_plane_bf16(const Plan &p, const float2 *d_x, const float *d_s
     const int64_t per = (n_items + ctas - 1) / ctas;
     const int64_t grid = (n_items + per - 1) / per;
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    k3_plane_tc<OpsBF16><<<(unsigned)grid, WS_THREADS, WS_SMEM, st>>>(
-        Y, reinterpret_cast<const uint4 *>(p.d_Gbf), reinterpret_cast<const uint4 *>(p.d_tcF),
-        p.d_tcTw, d_plane, p.K, p.nb, p.L, n_items, n_groups, per, nullptr, l1flag, p.nb / PEAK_CHUNK, mark_threshold(p),
-        p.d_status);
+    e = launch_after(early, k3_plane_tc<OpsBF16>, (unsigned)grid, WS_THREADS, WS_SMEM, st, Y, reinterpret_cast<const uint4 *>(p.d_Gbf),
+                     reinterpret_cast<const uint4 *>(p.d_tcF), p.d_tcTw, d_plane, p.K, p.nb, p.L, n_items, n_groups, per, nullptr,
+                     l1flag, p.nb / PEAK_CHUNK, mark_threshold(p), p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
     p.prof.launches += 2;
-    return cudaGetLastError();
+    return e;
 }
 
 // FP16-scaled ablation: scaled FP16 segment spectra, the FP16 bank (S G) and DFT image, FP32 plane.
 cudaError_t launch_plane_f16(const Plan &p, const float2 *d_x, const float *d_scale, char *ws, float *d_plane,
-                             cudaStream_t st, uint8_t *l1flag) {
+                             cudaStream_t st, uint8_t *l1flag, bool early) {
     if (p.S != TC_S_BF16 || !p.d_Gh || !p.d_tcFh) return cudaErrorInvalidValue;
     uint4 *Y = reinterpret_cast<uint4 *>(ws + p.ws_y);
     float *unscale = reinterpret_cast<float *>(ws + p.ws_segscale);
@@ -1035,10 +1035,10 @@ cudaError_t launch_plane_f16(const Plan &p, const float2 *d_x, const float *d_sc
     e = prepare_ws(k3_plane_tc<OpsF16>, WS_SMEM);
     if (e != cudaSuccess) return e;
     p.prof.begin(FDAS_STAGE_SEGMENTS, st);
-    k2_segments_f16<<<(unsigned)p.n_seg, TC_S_BF16 / 32, smem2, st>>>(d_x, d_scale, p.d_tw, Y, unscale,
-                                                                     (float)TC_S_BF16, p.nb, p.L, p.m / 2);
+    const int64_t n_zero16 = l1flag ? ((int64_t)p.K * (p.nb / PEAK_CHUNK) + 15) / 16 : 0;     // as in launch_plane_bf16
+    e = launch_after(early, k2_segments_f16, (unsigned)p.n_seg, TC_S_BF16 / 32, smem2, st, d_x, d_scale, p.d_tw, Y, unscale,
+                     (float)TC_S_BF16, p.nb, p.L, p.m / 2, reinterpret_cast<uint4 *>(l1flag), n_zero16);
     p.prof.end(FDAS_STAGE_SEGMENTS, st);
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int n_groups = (p.K + TC_G - 1) / TC_G;
     const int64_t n_items = p.n_seg * n_groups;
@@ -1047,15 +1047,13 @@ cudaError_t launch_plane_f16(const Plan &p, const float2 *d_x, const float *d_sc
     const int64_t ctas = std::min<int64_t>(n_items, (int64_t)sms);
     const int64_t per = (n_items + ctas - 1) / ctas;
     const int64_t grid = (n_items + per - 1) / per;
-    e = clear_marks(p, l1flag, st);
-    if (e != cudaSuccess) return e;
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    k3_plane_tc<OpsF16><<<(unsigned)grid, WS_THREADS, WS_SMEM, st>>>(
-        Y, reinterpret_cast<const uint4 *>(p.d_Gh), reinterpret_cast<const uint4 *>(p.d_tcFh), p.d_tcTw, d_plane,
-        p.K, p.nb, p.L, n_items, n_groups, per, unscale, l1flag, p.nb / PEAK_CHUNK, mark_threshold(p), p.d_status);
+    e = launch_after(early, k3_plane_tc<OpsF16>, (unsigned)grid, WS_THREADS, WS_SMEM, st, Y, reinterpret_cast<const uint4 *>(p.d_Gh),
+                     reinterpret_cast<const uint4 *>(p.d_tcFh), p.d_tcTw, d_plane, p.K, p.nb, p.L, n_items, n_groups, per, unscale,
+                     l1flag, p.nb / PEAK_CHUNK, mark_threshold(p), p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
     p.prof.launches += 2;
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace fdas
@@ -1080,11 +1078,10 @@ cudaError_t launch_plane_split(const Plan &p, const float2 *d_x, const float *d_
     const int64_t per = (n_items + ctas - 1) / ctas;
     const int64_t grid = (n_items + per - 1) / per;
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    k3_plane_tc_split<<<(unsigned)grid, WS_THREADS, SP_SMEM, st>>>(Y, p.d_G, reinterpret_cast<const uint4 *>(p.d_tcF), p.d_tcTw,
-                                                                   d_plane, p.K, p.nb, p.L, n_items, n_groups, per,
-                                                                   p.d_status);
+    e = launch_after(false, k3_plane_tc_split, (unsigned)grid, WS_THREADS, SP_SMEM, st, Y, p.d_G, reinterpret_cast<const uint4 *>(p.d_tcF),
+                     p.d_tcTw, d_plane, p.K, p.nb, p.L, n_items, n_groups, per, p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
     p.prof.launches += 1;
-    return cudaGetLastError();
+    return e;
 }
 }  // namespace fdas

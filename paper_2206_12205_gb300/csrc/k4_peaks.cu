@@ -517,8 +517,8 @@ __device__ __noinline__ uint32_t verify_dense(const E *__restrict__ plane, int64
 constexpr int DENSE_CELLS = 256;
 template <typename E>
 __device__ __forceinline__ void verify_unit(const E *__restrict__ plane, int64_t nb, int zmax, int K, bool anchored,
-                                            const UnitRef &ref, int64_t u, int32_t *__restrict__ unit_count,
-                                            uint32_t *__restrict__ unit_mask) {
+                                            const UnitRef &ref, int64_t u, int32_t *unit_count,
+                                            uint32_t *unit_mask) {
     const int lane = threadIdx.x & 31, H = ref.H;
     const uint32_t cells = lane < WORDS ? unit_mask[u * WORDS + lane] : 0u;
     int incl = __popc(cells);
@@ -683,9 +683,11 @@ __device__ __noinline__ void select_entry(int64_t k, const uint32_t *__restrict_
 // eight words, counts the entries kept before them (a few KB from L2) and writes its own in order.
 // Appended as the warps came by, the list was in random order (mean displacement 4000 of 13887) and
 // the search had lost the ray order's locality: N = 2^23, 85 templates, BF16.
-__global__ void __launch_bounds__(256) k4_compact(const uint32_t *__restrict__ keep, const uint32_t *__restrict__ order,
+__global__ void __launch_bounds__(256) k4_compact(const uint32_t *keep, const uint32_t *__restrict__ order,
                                                   int64_t n_order, uint32_t *__restrict__ work, unsigned int *__restrict__ count) {
     __shared__ unsigned int before[8], own[8];
+    grid_wait();
+    grid_release();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n_words = (n_order + 31) / 32, w0 = 8 * (int64_t)blockIdx.x, w = w0 + warp;
     unsigned int sum = 0;
@@ -723,6 +725,7 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32) k4_level1_marked(const E *_
                                                                     const uint32_t *__restrict__ order, int64_t n_order,
                                                                     LevelTable lt, int chunks2, uint32_t *__restrict__ work,
                                                                     uint32_t *__restrict__ keep) {
+    grid_release();
     const int lane = threadIdx.x & 31;
     if (blockIdx.x >= l1_blocks) {                   // block-uniform
         select_entry((int64_t)(blockIdx.x - l1_blocks) * blockDim.x + threadIdx.x, order, n_order, flags, zmax, K, lt,
@@ -810,6 +813,17 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_MIN_BLOCKS) k4_leve
     levels_group<E>(plane, nb, zmax, K, lt, chunks2, lt.lev[1].i_lo + blockIdx.y, c0, unit_count, unit_mask, l2mark);
 }
 
+// A word written by the kernel before a launch_after(early) one.
+__device__ __forceinline__ uint32_t ld_call(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Whether k4_levels_ordered may be launched early.
+template <typename E>
+constexpr bool EARLY_LEVELS = sizeof(E) == 2;
+
 // Level 2's region in the ray order of upload_levels_order, each entry a (row << 16 | chunk
 // group): block b takes the entries b, b + gridDim.x, ... (so the blocks in flight keep to a short
 // stretch of the order); with a persistent grid the next entry's code is loaded while the current
@@ -823,12 +837,20 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_MIN_BLOCKS) k4_leve
                                                                       int32_t *__restrict__ unit_count,
                                                                       uint32_t *__restrict__ unit_mask,
                                                                       const uint8_t *__restrict__ l2mark) {
-    if (d_count != nullptr) n_order = *d_count;   // a work list (the level-1 pass's selection blocks), written before this launch
+    // BF16 planes: launched early, the list read past the read-only path (ld_call).  FP32 planes' search
+    // stays as it was: with the wait it took 185 us instead of 170 (N = 2^23), wherever it was launched.
+    constexpr bool EARLY = EARLY_LEVELS<E>;
+    auto entry = [&](int64_t k) { return EARLY ? ld_call(order + k) : __ldg(order + k); };
+    if constexpr (EARLY) {
+        grid_wait();
+        grid_release();
+    }
+    if (d_count != nullptr) n_order = EARLY ? ld_call(d_count) : *d_count;   // a work list (the level-1 pass's selection blocks)
     int64_t idx = blockIdx.x;
-    uint32_t next = idx < n_order ? __ldg(order + idx) : 0u;
+    uint32_t next = idx < n_order ? entry(idx) : 0u;
     for (; idx < n_order; idx += gridDim.x) {
         const uint32_t o = next;
-        if (idx + gridDim.x < n_order) next = __ldg(order + idx + gridDim.x);
+        if (idx + gridDim.x < n_order) next = entry(idx + gridDim.x);
         if ((int)(o >> 16) >= lt.lev[1].rows) continue;                       // block-uniform
         const int c0 = ((int)(o & 0xffffu) * DETECT_WARPS + (threadIdx.x >> 5)) * CPW;
         if (c0 >= chunks2) continue;                                          // warp-uniform
@@ -948,8 +970,10 @@ constexpr int VERIFY_WARPS = 8;
 template <typename E>
 __global__ void __launch_bounds__(VERIFY_WARPS * 32, 4) k4_verify(const E *__restrict__ plane, int64_t nb, int zmax, int K,
                                                                LevelTable lt, const uint32_t *__restrict__ order,
-                                                               int64_t n_order, int32_t *__restrict__ unit_count,
-                                                               uint32_t *__restrict__ unit_mask) {
+                                                               int64_t n_order, int32_t *unit_count,
+                                                               uint32_t *unit_mask) {
+    grid_wait();
+    grid_release();
     const unsigned int *list = unit_list(unit_count);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int n = (int)*list;
@@ -998,7 +1022,7 @@ __global__ void __launch_bounds__(VERIFY_WARPS * 32, 4) k4_verify(const E *__res
 // per lane, the peaks dealt to the lanes in bin order (the order of the output within a unit).
 template <typename E>
 __device__ __noinline__ void emit_unit(const E *__restrict__ plane, int64_t nb, int zmax, bool anchored, UnitRef ref,
-                                       int64_t u, int64_t base, const uint32_t *__restrict__ unit_mask,
+                                       int64_t u, int64_t base, const uint32_t *unit_mask,
                                        fdas_peak *__restrict__ out, int max_peaks, uint32_t series) {
     const int lane = threadIdx.x & 31;
     const int H = ref.H;
@@ -1080,13 +1104,15 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t c, int32_t *warp_tot,
 // on the listed path) writes the total and the overflow flag.
 template <typename E>
 __global__ void __launch_bounds__(1024, 1) k4_emit_listed(const E *__restrict__ plane, int64_t nb, int zmax, LevelTable lt,
-                                                       int64_t n_units, const int32_t *__restrict__ unit_count,
-                                                       const uint32_t *__restrict__ unit_mask,
+                                                       int64_t n_units, const int32_t *unit_count,
+                                                       const uint32_t *unit_mask,
                                                        fdas_peak *__restrict__ out, int max_peaks, uint32_t series,
                                                        int32_t *__restrict__ npeaks, int32_t *__restrict__ status) {
     __shared__ uint32_t key[PEAK_LIST_CAP];
     __shared__ int32_t cnt[PEAK_LIST_CAP];
     __shared__ int32_t warp_tot[33];
+    grid_wait();
+    grid_release();
     const int t = threadIdx.x, warp = t >> 5;
     const unsigned int *list = unit_list(unit_count);
     const int n = (int)*list;
@@ -1171,7 +1197,7 @@ __global__ void __launch_bounds__(1024, 1) k4_emit_listed(const E *__restrict__ 
 
 template <typename E>
 cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks, int32_t *npeaks, uint32_t series,
-                      cudaStream_t st, const uint8_t *l1flag, bool list_cleared) {
+                      cudaStream_t st, const uint8_t *l1flag, bool list_cleared, bool early) {
     const LevelTable lt = make_levels(p);
     int32_t *unit_count = reinterpret_cast<int32_t *>(ws + p.ws_ucount);
     uint32_t *unit_mask = reinterpret_cast<uint32_t *>(ws + p.ws_umask);
@@ -1192,9 +1218,10 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
     // and so does the level search's work count (the next word); a search's long FFT has cleared
     // both already (list_cleared)
     uint32_t *list_hdr = reinterpret_cast<uint32_t *>(unit_count) - PEAK_LIST_WORDS;
+    cudaError_t e = cudaSuccess;
     if (!list_cleared) {
-        cudaError_t e0 = cudaMemsetAsync(list_hdr, 0, 3 * sizeof(uint32_t), st);
-        if (e0 != cudaSuccess) return e0;
+        e = cudaMemsetAsync(list_hdr, 0, 2 * sizeof(uint32_t), st);
+        if (e != cudaSuccess) return e;
     }
     p.prof.launches += lt.n_levels > 1 ? 3 : 2;
     // whether some level kernel leaves cells above the threshold to k4_verify
@@ -1218,7 +1245,8 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
             plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], !verify, n1, l1flag, unit_count, unit_mask, blocks, p.d_k4order, n_sel,
             lt, (int)chunks2, work, keep);
         if (keep) {
-            k4_compact<<<(unsigned)((p.k4order_n + 255) / 256), 256, 0, st>>>(keep, p.d_k4order, p.k4order_n, work, wcount);
+            e = launch_after(early, k4_compact, (unsigned)((p.k4order_n + 255) / 256), 256, 0, st, keep, p.d_k4order, p.k4order_n, work, wcount);
+            if (e != cudaSuccess) return e;
             p.prof.launches++;
         }
         p.prof.level1_fused++;
@@ -1254,9 +1282,11 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
             // skipped chunks cost one thread each instead of a warp's round trip in the search
             // (the work list from the level-1 pass's extra blocks, when the marks exist)
             const uint32_t *order = select_list ? work : p.d_k4order;
-            k4_levels_ordered<E><<<(unsigned)blocks, DETECT_WARPS * 32, 0, st>>>(
-                plane, p.nb, p.cfg.zmax, p.K, lt, (int)chunks2, order, p.k4order_n, wcount, unit_count,
-                unit_mask, l2mark);
+            // (the plane and the marks were complete when the kernel before, which waited or was launched
+            // plainly, let this one in; the work list is the last kernel's)
+            e = launch_after(early && EARLY_LEVELS<E>, k4_levels_ordered<E>, (unsigned)blocks, DETECT_WARPS * 32, 0, st, plane, p.nb, p.cfg.zmax, p.K, lt,
+                             (int)chunks2, order, p.k4order_n, wcount, unit_count, unit_mask, l2mark);
+            if (e != cudaSuccess) return e;
         } else {
             k4_levels<E><<<levels_grid, DETECT_WARPS * 32, 0, st>>>(plane, p.nb, p.cfg.zmax, p.K, lt, (int)chunks2,
                                                                      unit_count, unit_mask, l2mark);
@@ -1269,15 +1299,16 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
         const int64_t group = lt.anchored ? DETECT_WARPS : DETECT_WARPS * CPW;
         const int64_t n_order = (int64_t)lt.lev[1].rows * ((lt.lev[1].chunks + group - 1) / group);
         const uint32_t *order = !lt.anchored ? p.d_k4order : p.k4order_a_n == n_order ? p.d_k4order_a : nullptr;
-        k4_verify<E><<<(unsigned)std::max(1, 4 * sms_out), VERIFY_WARPS * 32, 0, st>>>(plane, p.nb, p.cfg.zmax, p.K, lt, order,
-                                                                                      n_order, unit_count, unit_mask);
+        e = launch_after(early, k4_verify<E>, (unsigned)std::max(1, 4 * sms_out), VERIFY_WARPS * 32, 0, st, plane, p.nb, p.cfg.zmax, p.K, lt,
+                         order, n_order, unit_count, unit_mask);
+        if (e != cudaSuccess) return e;
         p.prof.launches++;
     }
     // one block per SM: a listed unit per block and warp in the usual case, a range of all units each else
-    k4_emit_listed<E><<<(unsigned)std::max(1, sms_out), 1024, 0, st>>>(
-        plane, p.nb, p.cfg.zmax, lt, n_units, unit_count, unit_mask, peaks, p.cfg.max_peaks, series, npeaks, p.d_status);
+    e = launch_after(early, k4_emit_listed<E>, (unsigned)std::max(1, sms_out), 1024, 0, st, plane, p.nb, p.cfg.zmax, lt, n_units, unit_count,
+                     unit_mask, peaks, p.cfg.max_peaks, series, npeaks, p.d_status);
     p.prof.end(FDAS_STAGE_PEAKS, st);
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
@@ -1371,12 +1402,12 @@ cudaError_t upload_levels_order(Plan &p) {
 }
 
 cudaError_t launch_peaks(const Plan &p, const void *d_plane, bool bf16, char *ws, fdas_peak *d_peaks,
-                         int32_t *d_npeaks, uint32_t series, cudaStream_t st, const uint8_t *l1flag, bool list_cleared) {
+                         int32_t *d_npeaks, uint32_t series, cudaStream_t st, const uint8_t *l1flag, bool list_cleared, bool early) {
     if (bf16)
         return run_peaks<__nv_bfloat16>(p, reinterpret_cast<const __nv_bfloat16 *>(d_plane), ws, d_peaks, d_npeaks,
-                                        series, st, l1flag, list_cleared);
+                                        series, st, l1flag, list_cleared, early);
     return run_peaks<float>(p, reinterpret_cast<const float *>(d_plane), ws, d_peaks, d_npeaks, series, st, l1flag,
-                            list_cleared);
+                            list_cleared, early);
 }
 
 }  // namespace fdas
