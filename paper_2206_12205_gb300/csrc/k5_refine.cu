@@ -67,6 +67,7 @@
 
 #include "fdas_internal.cuh"
 #include "fresnel_table.cuh"
+#include "tap_range.cuh"
 
 namespace fdas {
 
@@ -538,9 +539,7 @@ __device__ Value64 eval64(const float2 *__restrict__ xhat, int64_t nb, int m, co
     const bool big = c.zz >= 1.0;
     const float dfar = FAR_C64 * fmaxf(1.f, sqrtf(zf));
     const int half = m / 2;
-    // folded offsets j with the tap inside the window: unfolded -half .. m - half - 1
-    const int64_t lo_k = c.k0 - half < 0 ? -c.k0 : -(int64_t)half;
-    const int64_t hi_k = c.k0 + (m - half) > nb ? nb - 1 - c.k0 : (int64_t)(m - half) - 1;
+    const TapRange on = taps_on_spectrum(c.k0, m, nb);                     // unfolded offsets
     cx<double> T0 = zero, T1 = zero, T2 = zero, SX = zero, SqX = zero;     // near taps, z >= 1
     int jl = 1, jh = 0;                                                    // near taps, z < 1
     if (!big) {
@@ -549,7 +548,7 @@ __device__ Value64 eval64(const float2 *__restrict__ xhat, int64_t nb, int m, co
     }
     for (int t = lane; t < m; t += 32) {
         const int ju = t - half;
-        if (ju < lo_k || ju > hi_k) continue;
+        if (ju < on.lo || ju > on.hi) continue;
         const int j = c.neg ? -ju : ju;
         if (j >= jl && j <= jh) continue;
         const float2 xv = __ldg(xhat + c.k0 + ju);
@@ -604,8 +603,8 @@ __device__ Value64 eval64(const float2 *__restrict__ xhat, int64_t nb, int m, co
     } else {
         // int_0^1 u^p exp(-i pi z u^2) sum_j X_j exp(2 pi i (j - dlt) u) du: lane l holds nodes +-x[l];
         // Horner over j from jh down to jl in exp(2 pi i u)
-        const int jlo = c.neg ? (int)max((int64_t)jl, -hi_k) : (int)max((int64_t)jl, lo_k);
-        const int jhi = c.neg ? (int)min((int64_t)jh, -lo_k) : (int)min((int64_t)jh, hi_k);
+        const TapRange near = taps_between(on, c.neg, jl, jh);
+        const int jlo = near.lo, jhi = near.hi;
         const double xg = gl.x[lane], wg = 0.5 * gl.w[lane];
         const double u0 = 0.5 * (1.0 - xg), u1 = 0.5 * (1.0 + xg);
         const cx<double> w0 = expipi64(2.0 * u0), w1 = expipi64(2.0 * u1);
