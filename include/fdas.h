@@ -223,10 +223,11 @@ fdas_status fdas_plane_static(fdas_plan_t plan, const float *d_xhat, void *d_pla
  * in row-major (i, r) order, or equal for later ones).  Peaks are written to d_peaks in
  * (harm, zi, r) order, at most max_peaks of them; *d_npeaks (device int32) receives the
  * true count, and a count above max_peaks also sets FDAS_DEV_PEAK_OVERFLOW.
- * The records are written from the list of (level, row, 512-bin chunk) units with cells above
- * their threshold, a unit to a warp; when there are more than 4096 (low thresholds) one block per
- * SM scans every unit's count instead (FP32 plane, N = 2^23, 85 templates, 11 million peaks:
- * 6.9 ms for the whole call, most of it the harmonic sums' local-maximum tests).
+ * The records are written from a list of (level, row, 512-bin chunk) units, a unit to a warp: the
+ * units that hold peaks, and on FP32 planes or with anchored sums those of levels 2 .. 16 with any
+ * cell above the threshold.  When there are more than 4096 (low thresholds) one block per SM
+ * scans every unit's count instead (FP32 plane, N = 2^23, 85 templates, 11 million peaks: 5.0 ms
+ * for the whole call, most of it the harmonic sums' local-maximum tests).
  * Errors: FDAS_E_INVALID, FDAS_E_STATE, FDAS_E_CUDA.
  */
 fdas_status fdas_peaks(fdas_plan_t plan, const void *d_plane, void *d_workspace,

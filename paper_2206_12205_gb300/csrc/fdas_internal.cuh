@@ -101,7 +101,8 @@ struct Plan {
 // (level, row, chunk) with a count and a PEAK_CHUNK-bit mask.
 constexpr int PEAK_ROWS = 8;
 constexpr int PEAK_CHUNK = 512;
-// The peak units with cells above their threshold, listed as the level kernels find them: a 4-word
+// The peak units that hold peaks, or whose cells the level kernels leave to k4_verify (any cell above
+// the threshold; such a unit may turn out to hold none), listed as they are found: a 4-word
 // header (the list's count, then the level search's work count) and up to PEAK_LIST_CAP unit numbers,
 // placed in the workspace directly before the unit counts.  When the list holds them all, the output
 // blocks share the listed units; else they scan every unit's count.  4096: the list and its counts

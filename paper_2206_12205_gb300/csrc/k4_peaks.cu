@@ -18,15 +18,15 @@
 // a span of whole sectors, where consecutive bins per lane would touch 32 sectors per load.  A
 // lane tests its 16 values against the threshold through their maximum; only cells above it (a
 // handful per plane, thousands with low thresholds) recompute their 3x3 neighbourhood's sums to
-// decide the peak: nine lanes of a warp to a cell (verify_unit), from the mask of such cells that the
-// level kernels leave; on BF16 planes level 1 and the plain sums' levels decide theirs in place
-// (IN_PLACE: what each way costs).
+// decide the peak.  Level 1, whose sums are plane values, decides its own (level1_unit), and on BF16
+// planes so do the plain sums' levels (IN_PLACE: what each way costs); the others leave the mask of such
+// cells to k4_verify, nine lanes of a warp to a cell or, where they are many, a lane to a bin.
 //
 // Output order (H, i, r): a "unit" is (level, row, chunk of CB bins), units are numbered in
 // that order, and
 //   pass A (k4_level1 over the plane, k4_levels over level 2's region, then k4_verify where cells
-//     were left to it) writes each unit's peak count and, when cells were above the threshold, its
-//     CB-bit mask, and lists those units (in no order);
+//     were left to it) writes each unit's peak count and CB-bit mask, and lists the units (in no
+//     order) that hold peaks, or whose cells were left to k4_verify;
 //   pass B (k4_emit_listed): when the list holds all of them (PEAK_LIST_CAP; the usual case) each
 //     listed unit goes to a warp, which sums the counts of the units before it and writes its
 //     records; otherwise every unit's count is scanned in order.  Either way a record's power is
@@ -53,7 +53,7 @@ constexpr int DETECT_WARPS = 4;          // warps per k4_level1 / k4_levels bloc
 constexpr int CPW = FDAS_K4_CPW;
 static_assert((CPW & (CPW - 1)) == 0 && CPW <= 2, "chunks per warp: 1 or 2 (chunks1 >= 2 is a power of two)");
 #ifndef FDAS_K4_L1_MIN_BLOCKS
-#define FDAS_K4_L1_MIN_BLOCKS 2          // resident k4_level1 blocks per SM the registers must allow
+#define FDAS_K4_L1_MIN_BLOCKS 8          // resident k4_level1 blocks per SM the registers must allow
 #endif
 #ifndef FDAS_K4_RAY_BF16
 #define FDAS_K4_RAY_BF16 1               // 1: the BF16 plane's levels in ray order too (the FP32 plane's always are)
@@ -278,8 +278,8 @@ __device__ __noinline__ bool local_max(const E *plane, int64_t nb, int zmax, int
     return true;
 }
 
-// The non-empty unit list of the step: PEAK_LIST_WORDS words directly before the counts (word 0
-// the number of non-empty units, words 4 .. the first PEAK_LIST_CAP unit numbers, in no order).
+// The unit list of the step: PEAK_LIST_WORDS words directly before the counts (word 0 the number of
+// units listed, words 4 .. the first PEAK_LIST_CAP unit numbers, in no order).
 __device__ __forceinline__ unsigned int *unit_list(int32_t *unit_count) {
     return reinterpret_cast<unsigned int *>(unit_count) - PEAK_LIST_WORDS;
 }
@@ -339,15 +339,6 @@ __device__ __forceinline__ void leave_sums(const float (&s)[LB], float thr, int 
     } else if (lane == 0) {
         unit_count[u] = 0;
     }
-}
-
-// The same from a lane's 16 consecutive bins (bit e of above: bin 16 lane + e).
-__device__ __forceinline__ void leave_runs(uint32_t above, int u, int32_t *__restrict__ unit_count,
-                                           uint32_t *__restrict__ unit_mask) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t lo = __shfl_sync(0xffffffffu, above, (2 * lane) & 31), hi = __shfl_sync(0xffffffffu, above, (2 * lane + 1) & 31);
-    if (__any_sync(0xffffffffu, above != 0)) leave_unit(lo | (hi << 16), u, unit_count, unit_mask);
-    else if (lane == 0) unit_count[u] = 0;
 }
 
 // One level H > 1 of one (row, chunk), lane bins rb + 32 e: S_H from S_{H/2}, then the unit's peaks or
@@ -568,32 +559,57 @@ __device__ __forceinline__ void verify_unit(const E *__restrict__ plane, int64_t
     if (lane < WORDS) unit_mask[u * WORDS + lane] = word;
 }
 
-// One level-1 unit u of row i, bins r0 .. r0 + 511, that holds a value above the threshold: its cells,
-// and, where nothing else needs k4_verify (IN_PLACE), its peaks.  Out of line, the values read again, so
-// that the stream over the plane keeps its registers.
+// The peaks of one level-1 unit u of row i, bins r0 .. r0 + 511, that holds a value above the threshold.  At
+// level 1 a neighbour's sum is a plane value, so a lane reads its 16 bins of the three rows as vectors (one
+// round trip for the whole unit, however many cells are above) and the bins beside them come by shuffles.
+// Out of line, the own row read again, so that the stream over the plane keeps its registers.
+// FP32, N = 2^23, 85 templates, 54 million peaks at all levels: 18.8 -> 11.0 ms with this in place of nine
+// lanes to a cell (below 256 cells a unit) or a lane to a bin.
 template <typename E>
-__device__ __noinline__ void level1_unit(const E *__restrict__ plane, int64_t nb, int zmax, int K, const LevelDesc &d, int i,
-                                         int64_t r0, int u, bool in_place, int32_t *__restrict__ unit_count,
-                                         uint32_t *__restrict__ unit_mask) {
-    typename Fmt<E>::Raw raw;
-    Fmt<E>::load_raw(plane + (int64_t)i * nb + r0 + LB * (threadIdx.x & 31), raw);
+__device__ __noinline__ void level1_unit(const E *__restrict__ plane, int64_t nb, int K, const LevelDesc &d, int i, int64_t r0,
+                                         int u, int32_t *__restrict__ unit_count, uint32_t *__restrict__ unit_mask) {
+    const int lane = threadIdx.x & 31;
+    const int64_t rl = r0 + LB * lane;
+    const E *own = plane + (int64_t)i * nb + rl;
+    typename Fmt<E>::Raw raw[3];                         // rows i, i - 1, i + 1
+    float edge[3];                                       // lane 0: the bin before the unit, lane 31: the bin after
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int a = (k == 2) - (k == 1);
+        edge[k] = -INFINITY;                             // an undefined neighbour: beaten by any cell above the threshold
+        if (i + a < 0 || i + a >= K) continue;
+        Fmt<E>::load_raw(own + a * nb, raw[k]);
+        if (lane == 0 && r0 > 0) edge[k] = ld_plane(own + a * nb, -1);
+        if (lane == 31 && rl + LB <= d.rmax) edge[k] = ld_plane(own + a * nb, LB);
+    }
     float v[LB];
-    Fmt<E>::widen(raw, v);
-    uint32_t above = 0;
+    Fmt<E>::widen(raw[0], v);
+    uint32_t pk = 0;
 #pragma unroll
     for (int e = 0; e < LB; e++)
-        if (v[e] > d.thr) above |= 1u << e;
-    leave_runs(above, u, unit_count, unit_mask);
-    // many cells: here, while the rows around are in the caches
-    if ((in_place && __any_sync(0xffffffffu, above != 0)) || (int)__reduce_add_sync(0xffffffffu, __popc(above)) >= DENSE_CELLS) {
-        __syncwarp();                                // the mask and the count of leave_runs, then their rewrite
-        UnitRef ref;
-        ref.H = 1;
-        ref.row = i;
-        ref.chunk = r0 / CB;
-        ref.rmax = d.rmax;
-        verify_unit<E>(plane, nb, zmax, K, false, ref, u, unit_count, unit_mask);
+        if (v[e] > d.thr) pk |= 1u << e;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        const int a = (k == 2) - (k == 1);
+        if (i + a < 0 || i + a >= K) continue;           // warp-uniform
+        float w[LB];
+        Fmt<E>::widen(raw[k], w);
+        float before = __shfl_up_sync(0xffffffffu, w[LB - 1], 1), after = __shfl_down_sync(0xffffffffu, w[0], 1);
+        if (lane == 0) before = edge[k];
+        if (lane == 31) after = edge[k];
+#pragma unroll
+        for (int e = 0; e < LB; e++) {
+            const float b = e == 0 ? before : w[e == 0 ? 0 : e - 1], c = e == LB - 1 ? after : w[e == LB - 1 ? e : e + 1];
+            const bool ok = (a <= 0 ? v[e] > b : v[e] >= b) && (a < 0 ? v[e] > w[e] : v[e] >= w[e]) && (a < 0 ? v[e] > c : v[e] >= c);
+            if (!ok) pk &= ~(1u << e);
+        }
     }
+    int cnt = __popc(pk);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    const uint32_t hi = __shfl_down_sync(0xffffffffu, pk, 1);
+    if (lane == 0) count_unit(unit_count, u, cnt);
+    if (cnt > 0 && !(lane & 1)) unit_mask[(int64_t)u * WORDS + (lane >> 1)] = pk | (hi << 16);
 }
 
 // Level 1 over the whole plane: a pure stream.  Grid (ceil(chunks1 / (DETECT_WARPS * CPW1)), K);
@@ -601,8 +617,8 @@ __device__ __noinline__ void level1_unit(const E *__restrict__ plane, int64_t nb
 // its 16 values through their maximum (BF16: packed) and widens them only when it holds a
 // candidate.  Few registers, so many warps keep the loads in flight.
 template <typename E>
-__global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_L1_MIN_BLOCKS) k4_level1(const E *__restrict__ plane, int64_t nb, int zmax,
-                                                              int K, LevelDesc d, int chunks1, bool in_place,
+__global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_L1_MIN_BLOCKS) k4_level1(const E *__restrict__ plane, int64_t nb, int K,
+                                                              LevelDesc d, int chunks1,
                                                               int32_t *__restrict__ unit_count,
                                                               uint32_t *__restrict__ unit_mask) {
     constexpr int CPW1 = Fmt<E>::EPV == 8 ? 4 : 2;
@@ -625,8 +641,7 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_L1_MIN_BLOCKS) k4_l
     }
     for (; hot; hot &= hot - 1) {
         const int c = c0 + __ffs(hot) - 1;
-        level1_unit<E>(plane, nb, zmax, K, d, i, (int64_t)c * CB, (int)d.unit0 + i * (int)d.chunks + c, in_place, unit_count,
-                       unit_mask);
+        level1_unit<E>(plane, nb, K, d, i, (int64_t)c * CB, (int)d.unit0 + i * (int)d.chunks + c, unit_count, unit_mask);
     }
 }
 
@@ -717,7 +732,7 @@ __global__ void __launch_bounds__(256) k4_compact(const uint32_t *keep, const ui
 // thread per entry of the block order; n_order = 0: none): the list depends only on the marks.
 template <typename E>
 __global__ void __launch_bounds__(DETECT_WARPS * 32) k4_level1_marked(const E *__restrict__ plane, int64_t nb, int zmax,
-                                                                    int K, LevelDesc d, bool in_place, int64_t n_units1,
+                                                                    int K, LevelDesc d, int64_t n_units1,
                                                                     const uint8_t *__restrict__ flags,
                                                                     int32_t *__restrict__ unit_count,
                                                                     uint32_t *__restrict__ unit_mask,
@@ -742,8 +757,7 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32) k4_level1_marked(const E *_
         const int64_t uu = u0 + (__ffs(todo) - 1);
         todo &= todo - 1;
         const int i = (int)(uu / d.chunks);
-        level1_unit<E>(plane, nb, zmax, K, d, i, (uu - (int64_t)i * d.chunks) * CB, (int)(d.unit0 + uu), in_place, unit_count,
-                       unit_mask);
+        level1_unit<E>(plane, nb, K, d, i, (uu - (int64_t)i * d.chunks) * CB, (int)(d.unit0 + uu), unit_count, unit_mask);
     }
 }
 
@@ -960,11 +974,10 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_MIN_BLOCKS) k4a_lev
     anch_chunk<E>(plane, nb, zmax, K, lt, (int)(o >> 16), c, unit_count, unit_mask);
 }
 
-// The units with cells above their threshold, one warp each: the listed ones, or, when they are more
-// than the list holds, every unit whose count is -1: level 1's in order, the others in the order of the
-// level search (order: entries row << 16 | chunk group, rows from lt.lev[1].i_lo; nullptr: column by
-// column), so that the sums around a unit's cells find their sectors in L2 (FP32, N = 2^23, 42 million
-// peaks: 37 ms in the units' order, 20 in the search's).  Four blocks to an SM at 64 registers: the
+// The units left to be tested (count -1), one warp each: those on the list, or, when it did not hold all
+// units, every one in the order of the level search (order: entries row << 16 | chunk group, rows from
+// lt.lev[1].i_lo; nullptr: column by column), so that the sums around a unit's cells find their sectors in
+// L2 (FP32, N = 2^23, 42 million peaks: 37 ms in the units' order, 20 in the search's).  Four blocks to an SM at 64 registers: the
 // gathers' latency is hidden by warps (anchored sums, N = 2^21, 19 million peaks: 13.8 ms with two, 12.0).
 constexpr int VERIFY_WARPS = 8;
 template <typename E>
@@ -981,23 +994,19 @@ __global__ void __launch_bounds__(VERIFY_WARPS * 32, 4) k4_verify(const E *__res
     if (n <= PEAK_LIST_CAP) {
         for (int k = (int)blockIdx.x + wid * (int)gridDim.x; k < n; k += VERIFY_WARPS * (int)gridDim.x) {
             const int64_t u = list[4 + k];
-            if (unit_count[u] >= 0) continue;            // tested in place
+            if (unit_count[u] >= 0) continue;            // level 1: tested already
             verify_unit<E>(plane, nb, zmax, K, anchored, unit_of(lt, u), u, unit_count, unit_mask);
         }
         return;
     }
-    const int64_t n1 = (int64_t)K * lt.lev[0].chunks, b1 = (n1 + 31) / 32;      // level 1: 32 units to a warp
     const int group = anchored ? DETECT_WARPS : DETECT_WARPS * CPW;             // chunks of an order's entry
-    const int64_t total = b1 + n_order * group;
+    const int64_t total = n_order * group;
     for (int64_t k = (int64_t)blockIdx.x * VERIFY_WARPS + wid; k < total; k += (int64_t)gridDim.x * VERIFY_WARPS) {
-        // the warp's up to 32 units, one per lane (level 1), or its chunk's levels 2 .. (lanes 1 .. 4)
-        int64_t u = -1;
-        if (k < b1) {
-            if (32 * k + lane < n1) u = 32 * k + lane;
-        } else if (lane > 0 && lane < lt.n_levels) {
-            const int64_t o = (k - b1) / group;
+        int64_t u = -1;                              // lanes 1 .. 4: the chunk's unit of that level
+        if (lane > 0 && lane < lt.n_levels) {
+            const int64_t o = k / group;
             const uint32_t code = order ? __ldg(order + o) : (uint32_t)(o % lt.lev[1].rows) << 16 | (uint32_t)(o / lt.lev[1].rows);
-            const int i = lt.lev[1].i_lo + (int)(code >> 16), c = (int)(code & 0xffffu) * group + (int)((k - b1) % group);
+            const int i = lt.lev[1].i_lo + (int)(code >> 16), c = (int)(code & 0xffffu) * group + (int)(k % group);
             int i_lo = 0, rows = 0;
             int64_t unit0 = 0, chunks = 0;
 #pragma unroll
@@ -1090,7 +1099,7 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t c, int32_t *warp_tot,
     return warp_tot[warp] + incl - c;
 }
 
-// The step's peaks, blocks of 1024 threads.  Usually the non-empty unit list holds every
+// The step's peaks, blocks of 1024 threads.  Usually the unit list holds every
 // non-empty unit (a handful to a few thousand of ~10^6): unit k of the list goes to warp k / grid of
 // block k mod grid, which sums the counts of the listed units with smaller numbers (its output
 // offset; the list and its counts in shared memory, 32 a step) and emits the unit's records.
@@ -1214,7 +1223,7 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
     // the plane kernel's unit marks (mark_threshold) bound the level-2 sums too
     const uint8_t *l2mark = l1flag && lt.n_levels > 1 ? l1flag : nullptr;
     p.prof.begin(FDAS_STAGE_PEAKS, st);
-    // the non-empty unit list starts empty (its counter: the word PEAK_LIST_WORDS before the counts)
+    // the unit list starts empty (its counter: the word PEAK_LIST_WORDS before the counts)
     // and so does the level search's work count (the next word); a search's long FFT has cleared
     // both already (list_cleared)
     uint32_t *list_hdr = reinterpret_cast<uint32_t *>(unit_count) - PEAK_LIST_WORDS;
@@ -1242,7 +1251,7 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
         const int64_t n_sel = select_list ? p.k4order_n : 0;
         const int64_t sel_blocks = (n_sel + DETECT_WARPS * 32 - 1) / (DETECT_WARPS * 32);
         k4_level1_marked<E><<<(unsigned)(blocks + sel_blocks), DETECT_WARPS * 32, 0, st>>>(
-            plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], !verify, n1, l1flag, unit_count, unit_mask, blocks, p.d_k4order, n_sel,
+            plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], n1, l1flag, unit_count, unit_mask, blocks, p.d_k4order, n_sel,
             lt, (int)chunks2, work, keep);
         if (keep) {
             e = launch_after(early, k4_compact, (unsigned)((p.k4order_n + 255) / 256), 256, 0, st, keep, p.d_k4order, p.k4order_n, work, wcount);
@@ -1251,8 +1260,7 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
         }
         p.prof.level1_fused++;
     } else {
-        k4_level1<E><<<level1_grid, DETECT_WARPS * 32, 0, st>>>(plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], (int)chunks1, !verify,
-                                                                 unit_count, unit_mask);
+        k4_level1<E><<<level1_grid, DETECT_WARPS * 32, 0, st>>>(plane, p.nb, p.K, lt.lev[0], (int)chunks1, unit_count, unit_mask);
     }
     p.prof.end(PROF_PEAKS_LEVEL1, st);
     if (lt.n_levels > 1 && lt.anchored) {
