@@ -226,7 +226,7 @@ fdas_status fdas_plane_static(fdas_plan_t plan, const float *d_xhat, void *d_pla
  * The records are written from a list of (level, row, 512-bin chunk) units, a unit to a warp: the
  * units that hold peaks, and on FP32 planes or with anchored sums those of levels 2 .. 16 with any
  * cell above the threshold.  When there are more than 4096 (low thresholds) one block per SM
- * scans every unit's count instead (FP32 plane, N = 2^23, 85 templates, 11 million peaks: 5.0 ms
+ * scans every unit's count instead (FP32 plane, N = 2^23, 85 templates, 11 million peaks: 4.7 ms
  * for the whole call, most of it the harmonic sums' local-maximum tests).
  * Errors: FDAS_E_INVALID, FDAS_E_STATE, FDAS_E_CUDA.
  */

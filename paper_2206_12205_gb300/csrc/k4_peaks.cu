@@ -1107,10 +1107,13 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t c, int32_t *warp_tot,
 // One block that sorted the list and emitted all units itself took 51 us for some 600 units of
 // anchored sums, this 6 us.
 // When more than PEAK_LIST_CAP units hold peaks (low thresholds, up to millions of peaks), every
-// block takes a contiguous range of units: it sums the counts before its range (its first output
+// block takes an equal share of the units: it sums the counts before its range (its first output
 // offset; a few MB read from L2 per block, no communication between blocks), then scans its
-// range 4096 units a round and emits the non-empty units as it goes.  The last block (or block 0
+// range, 4096 units a round at most, and deals the round's non-empty units to its warps.  Shares of
+// whole rounds left a plane of 10^4 units to two or three blocks (level 1 alone, FP32, N = 2^18, 27296 peaks:
+// 395 -> 55 us for the call; N = 2^16, 312797 peaks: 886 -> 35 us).  The last block (or block 0
 // on the listed path) writes the total and the overflow flag.
+static_assert(PEAK_LIST_CAP == 4 * 1024, "a round of the scan: four units a thread");
 template <typename E>
 __global__ void __launch_bounds__(1024, 1) k4_emit_listed(const E *__restrict__ plane, int64_t nb, int zmax, LevelTable lt,
                                                        int64_t n_units, const int32_t *unit_count,
@@ -1155,11 +1158,10 @@ __global__ void __launch_bounds__(1024, 1) k4_emit_listed(const E *__restrict__ 
         }
         writer = writer && warp == 31;
     } else {
-        // this block's units [ub, ue) (whole rounds of 4096) and the count before them
-        const int64_t rounds = (n_units + 4095) / 4096;
-        const int64_t per = (rounds + gridDim.x - 1) / gridDim.x;
-        const int64_t ub = min(n_units, (int64_t)blockIdx.x * per * 4096);
-        const int64_t ue = min(n_units, ub + per * 4096);
+        // this block's units [ub, ue), an equal share to every block, and the count before them
+        const int64_t per = (n_units + gridDim.x - 1) / gridDim.x;
+        const int64_t ub = min(n_units, (int64_t)blockIdx.x * per);
+        const int64_t ue = min(n_units, ub + per);
         writer = blockIdx.x == gridDim.x - 1 && warp == 0;
         {
             __shared__ unsigned long long pre_tot;       // counts are non-negative
@@ -1173,29 +1175,32 @@ __global__ void __launch_bounds__(1024, 1) k4_emit_listed(const E *__restrict__ 
             __syncthreads();
             total = (int64_t)pre_tot;
         }
-        for (int64_t u0 = ub; u0 < ue; u0 += 4 * 1024) {
-            const int64_t b0 = u0 + 4 * t;               // this thread's 4 units
-            int32_t v[4];
+        for (int64_t u0 = ub; u0 < ue; u0 += PEAK_LIST_CAP) {
+            const int n_round = (int)min((int64_t)PEAK_LIST_CAP, ue - u0);
+            int32_t v[4];                                // this thread's 4 units: counts, then offsets in the round
 #pragma unroll
-            for (int k = 0; k < 4; k++) v[k] = b0 + k < ue ? unit_count[b0 + k] : 0;
+            for (int k = 0; k < 4; k++) v[k] = 4 * t + k < n_round ? unit_count[u0 + 4 * t + k] : 0;
             int32_t tot;
             int32_t run = block_excl_scan(v[0] + v[1] + v[2] + v[3], warp_tot, &tot);
 #pragma unroll
             for (int k = 0; k < 4; k++) {
-                const int32_t mine = run;                // offset (in the round) of unit b0 + k
+                cnt[4 * t + k] = v[k];
+                key[4 * t + k] = (uint32_t)run;
                 run += v[k];
-                uint32_t busy = __ballot_sync(0xffffffffu, v[k] != 0);
-                while (busy) {                           // warp-uniform
-                    const int j = __ffs(busy) - 1;
-                    busy &= busy - 1;
-                    const int32_t off_j = __shfl_sync(0xffffffffu, mine, j);
-                    const int64_t u = u0 + 4 * (32 * warp + j) + k;
-                    emit_unit<E>(plane, nb, zmax, lt.anchored != 0, unit_of(lt, u), u, total + off_j, unit_mask, out, max_peaks,
-                                 series);
+            }
+            __syncthreads();
+            // unit j to warp (j - j / 32) mod 32: neighbours to different warps, a warp's 32 counts on 32 banks
+            const int lane = t & 31;
+            for (int j0 = 0; j0 < n_round; j0 += 1024) {
+                uint32_t busy = __ballot_sync(0xffffffffu, cnt[j0 + 32 * lane + ((warp + lane) & 31)] != 0);
+                for (; busy; busy &= busy - 1) {         // warp-uniform
+                    const int l = __ffs(busy) - 1, j = j0 + 32 * l + ((warp + l) & 31);
+                    emit_unit<E>(plane, nb, zmax, lt.anchored != 0, unit_of(lt, u0 + j), u0 + j, total + key[j], unit_mask, out,
+                                 max_peaks, series);
                 }
             }
             total += tot;
-            __syncthreads();                             // warp_tot is reused by the next round
+            __syncthreads();                             // the arrays are reused by the next round
         }
     }
     if (writer && (t & 31) == 0) {
