@@ -757,7 +757,13 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32) k4_level1_marked(const E *_
         const int64_t uu = u0 + (__ffs(todo) - 1);
         todo &= todo - 1;
         const int i = (int)(uu / d.chunks);
-        level1_unit<E>(plane, nb, K, d, i, (uu - (int64_t)i * d.chunks) * CB, (int)(d.unit0 + uu), unit_count, unit_mask);
+        const int64_t r0 = (uu - (int64_t)i * d.chunks) * CB;
+        typename Fmt<E>::Raw raw;                    // most are marked for level 2's sake (mark_threshold)
+        Fmt<E>::load_raw(plane + (int64_t)i * nb + r0 + LB * lane, raw);
+        if (__any_sync(0xffffffffu, Fmt<E>::max16(raw) > d.thr))
+            level1_unit<E>(plane, nb, K, d, i, r0, (int)(d.unit0 + uu), unit_count, unit_mask);
+        else if (lane == 0)
+            unit_count[d.unit0 + uu] = 0;
     }
 }
 
