@@ -297,7 +297,7 @@ fdas_status fdas_peaks(fdas_plan_t plan, const void *d_plane, void *d_workspace,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     p->prof.calls++;
     cudaError_t e = fdas::launch_peaks(*p, d_plane, plane_is_bf16(p), static_cast<char *>(d_workspace), d_peaks,
-                                       d_npeaks, 0u, st);
+                                       d_npeaks, 0u, st, nullptr, false, false, true);
     return record(p, e);
 }
 
@@ -323,7 +323,7 @@ fdas_status fdas_search(fdas_plan_t plan, const float *d_series, void *d_workspa
     uint8_t *l1flag = fdas::level1_fusable(*p) ? reinterpret_cast<uint8_t *>(ws + p->ws_l1flag) : nullptr;
     if (e == cudaSuccess) e = launch_plane_any(p, x, scale, ws, d_plane, st, l1flag, early);
     if (e == cudaSuccess)
-        e = fdas::launch_peaks(*p, d_plane, plane_is_bf16(p), ws, d_peaks, d_npeaks, 0u, st, l1flag, true, early);
+        e = fdas::launch_peaks(*p, d_plane, plane_is_bf16(p), ws, d_peaks, d_npeaks, 0u, st, l1flag, true, early, true);
     return record(p, e);
 }
 

@@ -142,6 +142,10 @@ void gauss_legendre(int n, double *xs, double *ws);
 // costs more than the gap (BF16, N = 2^20: 116 -> 123 us; N = 2^23: 588 -> 608 us), and in batches blocks that wait keep the
 // other lanes' out (12 series of 2^21, 3 lanes: 3.32 -> 3.52 ms); these launch plainly, which makes
 // both calls no-ops.
+//   early_tail: the peak search's list and output kernels (k4_compact, k4_verify, k4_emit_listed) in a call
+// by itself, of any size.  They wait for little, and what they save is the gap: k4_verify and k4_compact,
+// launched plainly, had made calls with few peaks slower than one kernel that did it all (fdas_peaks, FP32,
+// N = 2^16: 21.8 us once, 24.8 -> 20.1; search, FP16, N = 2^20, 21 templates: 69.9 once, 71.8 -> 66).
 inline int64_t launch_early_bins(int device) {
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device >= 0 ? device : 0);
@@ -214,10 +218,12 @@ bool levels_order(const Plan &p, std::vector<uint32_t> &order, bool anchored = f
 int64_t levels_order_size(const Plan &p);   // entries of the plain order (level 2's region)
 cudaError_t upload_levels_order(Plan &p);
 // list_cleared: the peak list's counters (PEAK_LIST_WORDS before the unit counts) were cleared
-// earlier on the stream (launch_spectrum does); else the peak search clears them itself.
+// earlier on the stream (launch_spectrum does); else the peak search clears them itself.  early,
+// early_tail: see launch_after.
 cudaError_t launch_peaks(const Plan &p, const void *d_plane, bool bf16, char *ws,
                          fdas_peak *d_peaks, int32_t *d_npeaks, uint32_t series, cudaStream_t st,
-                         const uint8_t *l1flag = nullptr, bool list_cleared = false, bool early = false);
+                         const uint8_t *l1flag = nullptr, bool list_cleared = false, bool early = false,
+                         bool early_tail = false);
 cudaError_t launch_band_max(const Plan &p, const void *d_plane, bool bf16, const int64_t *d_lo, const int64_t *d_hi,
                             int n_bands, int64_t max_width, unsigned long long *d_slot, float *d_value,
                             int64_t *d_r, int32_t *d_zi, cudaStream_t st);

@@ -1217,7 +1217,7 @@ __global__ void __launch_bounds__(1024, 1) k4_emit_listed(const E *__restrict__ 
 
 template <typename E>
 cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks, int32_t *npeaks, uint32_t series,
-                      cudaStream_t st, const uint8_t *l1flag, bool list_cleared, bool early) {
+                      cudaStream_t st, const uint8_t *l1flag, bool list_cleared, bool early, bool early_tail) {
     const LevelTable lt = make_levels(p);
     int32_t *unit_count = reinterpret_cast<int32_t *>(ws + p.ws_ucount);
     uint32_t *unit_mask = reinterpret_cast<uint32_t *>(ws + p.ws_umask);
@@ -1265,7 +1265,7 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
             plane, p.nb, p.cfg.zmax, p.K, lt.lev[0], n1, l1flag, unit_count, unit_mask, blocks, p.d_k4order, n_sel,
             lt, (int)chunks2, work, keep);
         if (keep) {
-            e = launch_after(early, k4_compact, (unsigned)((p.k4order_n + 255) / 256), 256, 0, st, keep, p.d_k4order, p.k4order_n, work, wcount);
+            e = launch_after(early_tail, k4_compact, (unsigned)((p.k4order_n + 255) / 256), 256, 0, st, keep, p.d_k4order, p.k4order_n, work, wcount);
             if (e != cudaSuccess) return e;
             p.prof.launches++;
         }
@@ -1318,13 +1318,13 @@ cudaError_t run_peaks(const Plan &p, const E *plane, char *ws, fdas_peak *peaks,
         const int64_t group = lt.anchored ? DETECT_WARPS : DETECT_WARPS * CPW;
         const int64_t n_order = (int64_t)lt.lev[1].rows * ((lt.lev[1].chunks + group - 1) / group);
         const uint32_t *order = !lt.anchored ? p.d_k4order : p.k4order_a_n == n_order ? p.d_k4order_a : nullptr;
-        e = launch_after(early, k4_verify<E>, (unsigned)std::max(1, 4 * sms_out), VERIFY_WARPS * 32, 0, st, plane, p.nb, p.cfg.zmax, p.K, lt,
+        e = launch_after(early_tail, k4_verify<E>, (unsigned)std::max(1, 4 * sms_out), VERIFY_WARPS * 32, 0, st, plane, p.nb, p.cfg.zmax, p.K, lt,
                          order, n_order, unit_count, unit_mask);
         if (e != cudaSuccess) return e;
         p.prof.launches++;
     }
     // one block per SM: a listed unit per block and warp in the usual case, a range of all units each else
-    e = launch_after(early, k4_emit_listed<E>, (unsigned)std::max(1, sms_out), 1024, 0, st, plane, p.nb, p.cfg.zmax, lt, n_units, unit_count,
+    e = launch_after(early_tail, k4_emit_listed<E>, (unsigned)std::max(1, sms_out), 1024, 0, st, plane, p.nb, p.cfg.zmax, lt, n_units, unit_count,
                      unit_mask, peaks, p.cfg.max_peaks, series, npeaks, p.d_status);
     p.prof.end(FDAS_STAGE_PEAKS, st);
     return e != cudaSuccess ? e : cudaGetLastError();
@@ -1421,12 +1421,12 @@ cudaError_t upload_levels_order(Plan &p) {
 }
 
 cudaError_t launch_peaks(const Plan &p, const void *d_plane, bool bf16, char *ws, fdas_peak *d_peaks,
-                         int32_t *d_npeaks, uint32_t series, cudaStream_t st, const uint8_t *l1flag, bool list_cleared, bool early) {
+                         int32_t *d_npeaks, uint32_t series, cudaStream_t st, const uint8_t *l1flag, bool list_cleared, bool early, bool early_tail) {
     if (bf16)
         return run_peaks<__nv_bfloat16>(p, reinterpret_cast<const __nv_bfloat16 *>(d_plane), ws, d_peaks, d_npeaks,
-                                        series, st, l1flag, list_cleared, early);
+                                        series, st, l1flag, list_cleared, early, early_tail);
     return run_peaks<float>(p, reinterpret_cast<const float *>(d_plane), ws, d_peaks, d_npeaks, series, st, l1flag,
-                            list_cleared, early);
+                            list_cleared, early, early_tail);
 }
 
 }  // namespace fdas
