@@ -151,6 +151,16 @@ inline int64_t launch_early_bins(int device) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device >= 0 ? device : 0);
     return (int64_t)sms * 2048;                      // N = 2^19 on 152 SMs
 }
+// Whether the second FFT pass and the BF16 segment FFTs let the next kernel's blocks in at once, or only as
+// their own blocks exit (which still saves the launch).  Blocks that are in and wait hold shared memory and
+// registers that this kernel's last waves, or other streams' kernels, could use.  Before k3_plane_tc, whose
+// blocks take an SM each, that costs more than it saves above 1024 bins per SM (N = 2^19, 85 templates, BF16, us a
+// search, plain launches / early and in at once / at exit: one stream 81.3 / 73.2 / 67.6, four 46.7 / 48.2 / 47.2,
+// eight 42.5 / 44.2 / 42.4); up to there, and before the FP32 plane kernel, it saves (N = 2^19, FP32, one
+// stream: 133.8 / 115.9 / 121; eight streams 82.8 / 86.2 / 82).
+inline bool release_at_once(const Plan &p) {
+    return (p.cfg.precision != FDAS_BF16 && p.cfg.precision != FDAS_FP16_SCALED) || 2 * p.nb <= launch_early_bins(p.device);
+}
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... P, typename... A>

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(2 * k1_groups_b(M2) * (M2 / 32), FDAS_K1B_MIN_
                                                                          double *partial, int M1,
                                                                          unsigned int *__restrict__ ticket, int64_t nb,
                                                                          double sigma2_fixed, double *__restrict__ sigma2_out,
-                                                                         float *__restrict__ scale_out) {
+                                                                         float *__restrict__ scale_out, bool release) {
     constexpr int T = M2 / 32, C2 = k1_groups_b(M2), G = 2 * C2;
     constexpr int E = k1_region(M2, G);
     extern __shared__ float2 smb[];       // G * E entries
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(2 * k1_groups_b(M2) * (M2 / 32), FDAS_K1B_MIN_
     __shared__ float2 w64[32];            // W_N^{M1 T i} = W_64^i
     for (int i = threadIdx.x; i < 32; i += G * T) w64[i] = twN(lo, hi, (int64_t)M1 * T * i);
     grid_wait();
-    grid_release();
+    if (release) grid_release();
     float2 v[32];
 #pragma unroll
     for (int i = 0; i < 32; i++) v[i] = B[(int64_t)row * M2 + t + i * T];
@@ -261,7 +261,7 @@ cudaError_t run_pass_b(const Plan &p, const float2 *B, float2 *X, double *partia
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return launch_after(early, kern, p.M1 / (2 * C2), 2 * C2 * (M2 / 32), smem, st, B, p.d_tw, p.d_twn_lo, p.d_twn_hi, X, partial, p.M1,
-                        ticket, p.nb, p.cfg.sigma2, sigma2, scale);
+                        ticket, p.nb, p.cfg.sigma2, sigma2, scale, release_at_once(p));
 }
 
 }  // namespace

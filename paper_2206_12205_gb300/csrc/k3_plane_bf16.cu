@@ -85,13 +85,13 @@ __global__ void __launch_bounds__(TC_S_BF16 / 32) k2_segments_bf16(const float2 
                                                                    const float2 *__restrict__ tw,
                                                                    uint4 *__restrict__ Y, int64_t nb, int L,
                                                                    int half_m, uint4 *__restrict__ zero16,
-                                                                   int64_t n_zero16) {
+                                                                   int64_t n_zero16, bool release) {
     constexpr int S = TC_S_BF16, T = S / 32;
     extern __shared__ float2 sm[];
     const int t = threadIdx.x;
     const int64_t j = blockIdx.x;
     grid_wait();
-    grid_release();
+    if (release) grid_release();
     for (int64_t w = j * T + t; w < n_zero16; w += (int64_t)gridDim.x * T) zero16[w] = make_uint4(0u, 0u, 0u, 0u);
     const float scale = scale_ptr ? *scale_ptr : 1.0f;
     const int64_t base = j * L - half_m;
@@ -1004,7 +1004,7 @@ cudaError_t launch_plane_bf16(const Plan &p, const float2 *d_x, const float *d_s
     const int64_t n_zero16 = l1flag ? ((int64_t)p.K * (p.nb / PEAK_CHUNK) + 15) / 16 : 0;
     p.prof.begin(FDAS_STAGE_SEGMENTS, st);
     e = launch_after(early, k2_segments_bf16, (unsigned)p.n_seg, TC_S_BF16 / 32, smem2, st, d_x, d_scale, p.d_tw, Y, p.nb, p.L, p.m / 2,
-                     reinterpret_cast<uint4 *>(l1flag), n_zero16);
+                     reinterpret_cast<uint4 *>(l1flag), n_zero16, release_at_once(p));
     p.prof.end(FDAS_STAGE_SEGMENTS, st);
     if (e != cudaSuccess) return e;
     const int n_groups = (p.K + TC_G - 1) / TC_G;
