@@ -203,7 +203,9 @@ __global__ void k1_apply_scale(const float2 *__restrict__ X, const float *__rest
 // the top: the median's next bit is set when no more than `rank` values lie below the prefix with
 // it set.  31 counts of the block's values, each a compare per value and one barrier, in place of
 // the 78 compare-exchange passes of a bitonic sort of 4096 powers through shared memory: N = 2^21,
-// blocks of 4096: 43 -> 13 us.
+// blocks of 4096: 43 -> 13 us.  Blocks of 32768 and 65536 give a thread 32 and 64 powers at 64 registers (1024
+// threads): those two spill (240 and 948 bytes) and are still ahead of the sort (N = 2^18, blocks of 32768, whole
+// call: 361 -> 86 us; blocks of 65536 did not fit it).
 template <int PER>
 __global__ void __launch_bounds__(1024) k1_local_norm(const float2 *__restrict__ X, float2 *__restrict__ out, int B) {
     __shared__ int part[2][32];
@@ -310,12 +312,14 @@ cudaError_t launch_spectrum(const Plan &p, const float *d_series, char *ws, cuda
 cudaError_t launch_local_norm(const Plan &p, const float2 *d_x, float2 *d_out, cudaStream_t st) {
     const int B = p.cfg.norm_block;
     if (B <= 0 || p.nb % B != 0) return cudaErrorInvalidValue;
-    // 16 values a thread between 512 and 16384 bins (fewer, larger blocks of threads outside)
+    // 16 values a thread between 1024 and 16384 bins (fewer, larger blocks of threads outside; with 512 bins one
+    // warp a block counted too long: N = 2^18, whole call 34.7 us, with two warps 30.4, the sort 32.9)
     const unsigned blocks = (unsigned)(p.nb / B);
     switch (B) {
         case 64: k1_local_norm<2><<<blocks, 32, 0, st>>>(d_x, d_out, B); break;
         case 128: k1_local_norm<4><<<blocks, 32, 0, st>>>(d_x, d_out, B); break;
         case 256: k1_local_norm<8><<<blocks, 32, 0, st>>>(d_x, d_out, B); break;
+        case 512: k1_local_norm<8><<<blocks, 64, 0, st>>>(d_x, d_out, B); break;
         case 32768: k1_local_norm<32><<<blocks, 1024, 0, st>>>(d_x, d_out, B); break;
         case 65536: k1_local_norm<64><<<blocks, 1024, 0, st>>>(d_x, d_out, B); break;
         default: k1_local_norm<16><<<blocks, B / 16, 0, st>>>(d_x, d_out, B); break;
