@@ -279,8 +279,8 @@ fdas_status fdas_get_templates(fdas_plan_t plan, float *d_out, void *stream);
 
 /*
  * Failure-detection self-check of the bounded waits.  Launches one block on the stream whose
- * thread waits on an mbarrier that nothing arrives on, in the bounded form every wait of the
- * plane kernels has, for at most max_cycles SM clock cycles (1 .. 2^36; at 2 GHz 2e9 is about
+ * warp waits on an mbarrier that nothing arrives on, in the bounded form the plane kernels'
+ * waits have, for at most max_cycles SM clock cycles (1 .. 2^36; at 2 GHz 2e9 is about
  * one second).  When the bound runs out the block sets FDAS_DEV_TIMEOUT in the plan's status
  * word and returns, leaving the context usable; read it with fdas_device_status.  Needs
  * fdas_make_templates first (the status word).  Errors: FDAS_E_INVALID, FDAS_E_STATE,

@@ -47,14 +47,18 @@ bool args_aligned(const void *series, const void *xhat, const void *ws, const vo
 }  // namespace
 
 namespace fdas {
-// One thread waits on a fresh mbarrier (phase 0 completes only on an arrival that never comes)
-// for at most max_cycles, then records the timeout: the bounded wait of the plane kernels.
+// One warp waits on a fresh mbarrier (phase 0 completes only on an arrival that never comes) for at
+// most max_cycles, then records the timeout: the bounded wait of the plane kernels.
 __global__ void wait_check(int64_t max_cycles, int32_t *status) {
     __shared__ uint64_t bar;
+    __shared__ int abort_flag;
     if (threadIdx.x == 0) {
         tc::mbar_init(&bar, 1);
-        if (!tc::mbar_wait_bounded(&bar, 0, (long long)max_cycles)) atomicOr(status, FDAS_DEV_TIMEOUT);
+        abort_flag = 0;
     }
+    __syncwarp();
+    const bool got = tc::mbar_wait_warp(&bar, 0, (long long)max_cycles, &abort_flag);
+    if (threadIdx.x == 0 && !got) atomicOr(status, FDAS_DEV_TIMEOUT);
 }
 
 cudaError_t launch_plane_any(const Plan &p, const float2 *x, const float *scale, char *ws, void *d_plane,

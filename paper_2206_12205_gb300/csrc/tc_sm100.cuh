@@ -63,6 +63,22 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
     return true;
 }
 
+// The bounded wait of a whole warp, given up by all of its lanes or none: what follows is a .sync.aligned
+// TMEM access or MMA, which part of a warp must not reach.  It ends when every lane has seen the phase
+// complete, when max_cycles have passed (then *abort_flag is set), or when another warp has set *abort_flag.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, long long max_cycles, volatile int *abort_flag) {
+    bool done = mbar_try_wait(bar, parity);
+    if (__all_sync(0xffffffffu, done)) return true;
+    const long long t0 = clock64();
+    while (true) {
+        done = done || mbar_try_wait(bar, parity);
+        if (__all_sync(0xffffffffu, done)) return true;
+        const bool late = clock64() - t0 > max_cycles;
+        if (late) *abort_flag = 1;
+        if (__any_sync(0xffffffffu, late || *abort_flag != 0)) return false;
+    }
+}
+
 // ---------------------------------------------------------------- TMEM
 // Allocate ncols (power of two >= 32) TMEM columns; the whole warp executes it; the TMEM
 // address is written to *dst (shared memory).
