@@ -126,21 +126,13 @@ struct FresnelSpot {
     int idx;
     float centre;
 };
-__host__ __device__ __forceinline__ FresnelSpot fresnel_spot(float x) {
+__device__ __forceinline__ FresnelSpot fresnel_spot(float x) {
     if (x < 8.f) {
         const int i = (int)(x * 16.f);
         return {i, ((float)i + 0.5f) * 0.0625f};
     }
-    unsigned b = 0;
-#ifdef __CUDA_ARCH__
-    b = __float_as_uint(x);
+    const unsigned b = __float_as_uint(x);
     const float centre = __uint_as_float((b & 0xFFF80000u) | 0x00040000u);
-#else
-    __builtin_memcpy(&b, &x, 4);
-    const unsigned cb = (b & 0xFFF80000u) | 0x00040000u;
-    float centre = 0.f;
-    __builtin_memcpy(&centre, &cb, 4);
-#endif
     const int i = (int)(b >> 19) - (130 << 4);      // exponent 130: 8 <= x < 16
     return {FRESNEL_UNIFORM + (i < 127 ? i : 127), centre};
 }

@@ -619,7 +619,7 @@ __device__ __forceinline__ bool sp_wait(uint64_t *bar, uint32_t parity, volatile
     return tc::mbar_wait_warp(bar, parity, WAIT_CYCLES, abort_flag);
 }
 
-__global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 *Y,
+__global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 *__restrict__ Y,
                                                                    const float2 *__restrict__ G,
                                                                    const uint4 *__restrict__ Fimg,
                                                                    const float2 *__restrict__ tw,
@@ -662,8 +662,6 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 
     tc::fence_before_thread_sync();
     __syncthreads();
     tc::fence_after_thread_sync();
-    grid_wait();
-    grid_release();
 
     const uint32_t tbase = *tslot;
     const int64_t it0 = (int64_t)blockIdx.x * items_per_cta;
@@ -754,7 +752,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc_split(const float2 
             const float2 *Gp = G + (int64_t)(z < K ? z : 0) * TC_S_BF16 + (32 * hp + 8 * i) * TC_R + n2;
 #pragma unroll
             for (int e = 0; e < 8; e++) {
-                y[e] = Yp[e * TC_R];
+                y[e] = __ldg(Yp + e * TC_R);
                 g[e] = __ldg(Gp + e * TC_R);
             }
         };
@@ -1083,10 +1081,10 @@ cudaError_t launch_plane_split(const Plan &p, const float2 *d_x, const float *d_
     const int64_t per = (n_items + ctas - 1) / ctas;
     const int64_t grid = (n_items + per - 1) / per;
     p.prof.begin(FDAS_STAGE_CORRELATE, st);
-    e = launch_after(false, k3_plane_tc_split, (unsigned)grid, WS_THREADS, SP_SMEM, st, Y, p.d_G, reinterpret_cast<const uint4 *>(p.d_tcF),
-                     p.d_tcTw, d_plane, p.K, p.nb, p.L, n_items, n_groups, per, p.d_status);
+    k3_plane_tc_split<<<(unsigned)grid, WS_THREADS, SP_SMEM, st>>>(Y, p.d_G, reinterpret_cast<const uint4 *>(p.d_tcF), p.d_tcTw,
+                                                                   d_plane, p.K, p.nb, p.L, n_items, n_groups, per, p.d_status);
     p.prof.end(FDAS_STAGE_CORRELATE, st);
     p.prof.launches += 1;
-    return e;
+    return cudaGetLastError();
 }
 }  // namespace fdas

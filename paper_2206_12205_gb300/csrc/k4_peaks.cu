@@ -96,24 +96,6 @@ struct Fmt<float> {
         for (int k = 0; k < LB / 4; k++) m = fmaxf(fmaxf(m, fmaxf(r.v[k].x, r.v[k].y)), fmaxf(r.v[k].z, r.v[k].w));
         return m;
     }
-    __device__ __forceinline__ static void load(const float *p, float (&o)[4]) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
-        o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-    }
-    __device__ __forceinline__ static float load16(const float *p, float (&s)[LB]) {
-        float m = -INFINITY;
-#pragma unroll
-        for (int k = 0; k < LB / 4; k++) {
-            float v[4];
-            load(p + 4 * k, v);
-#pragma unroll
-            for (int e = 0; e < 4; e++) {
-                s[4 * k + e] = v[e];
-                m = fmaxf(m, v[e]);
-            }
-        }
-        return m;
-    }
 };
 template <>
 struct Fmt<__nv_bfloat16> {
@@ -139,28 +121,6 @@ struct Fmt<__nv_bfloat16> {
         __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162 *>(&w[0]);
 #pragma unroll
         for (int k = 1; k < 8; k++) m = __hmax2(m, *reinterpret_cast<const __nv_bfloat162 *>(&w[k]));
-        return fmaxf(__low2float(m), __high2float(m));
-    }
-    __device__ __forceinline__ static void load(const __nv_bfloat16 *p, float (&o)[8]) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            o[2 * k] = __uint_as_float(w[k] << 16);
-            o[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
-        }
-    }
-    __device__ __forceinline__ static float load16(const __nv_bfloat16 *p, float (&s)[LB]) {
-        const uint4 a = __ldg(reinterpret_cast<const uint4 *>(p));
-        const uint4 b = __ldg(reinterpret_cast<const uint4 *>(p + 8));
-        const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162 *>(&w[0]);
-#pragma unroll
-        for (int k = 0; k < 8; k++) {
-            m = __hmax2(m, *reinterpret_cast<const __nv_bfloat162 *>(&w[k]));
-            s[2 * k] = __uint_as_float(w[k] << 16);
-            s[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
-        }
         return fmaxf(__low2float(m), __high2float(m));
     }
 };
