@@ -18,7 +18,7 @@
 // a span of whole sectors, where consecutive bins per lane would touch 32 sectors per load.  A
 // lane tests its 16 values against the threshold through their maximum; only cells above it (a
 // handful per plane, thousands with low thresholds) recompute their 3x3 neighbourhood's sums to
-// decide the peak.  Level 1, whose sums are plane values, decides its own (level1_unit), and on BF16
+// decide the peak.  Level 1, whose sums are plane values, decides its own (level1_many), and on BF16
 // planes so do the plain sums' levels (IN_PLACE: what each way costs); the others leave the mask of such
 // cells to k4_verify, nine lanes of a warp to a cell or, where they are many, a lane to a bin.
 //
@@ -32,7 +32,7 @@
 //     records; otherwise every unit's count is scanned in order.  Either way a record's power is
 //     S_H recomputed at its cell, at offset + rank.
 // Listed calls with thousands of peaks (FP32 plane, N = 2^21, 85 templates, low thresholds, some 3000
-// units): 260 -> 139 us, of which the tests were 50 and the output 75.
+// units): 243-260 us with each lane testing its own cells and one block writing all records, 134 now.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -414,9 +414,7 @@ __device__ __forceinline__ UnitRef unit_of(const LevelTable &lt, int64_t u) {
 // The mask of a unit's peaks (lane w < 16: word w) among its cells when they are many: a lane to a bin,
 // 32 consecutive bins at a time, so that the gathers of a warp share their sectors.  Every lane's own
 // sum serves its row neighbours through shuffles; then the cells still standing look at the rows
-// before and after, each lane up to the first neighbour that beats its cell.  With every second cell of
-// an FP32 plane above the threshold (N = 2^23, 54 million peaks) the whole call takes 19.8 ms, in place
-// 20.3 and nine lanes to a cell 71.
+// before and after, each lane up to the first neighbour that beats its cell.
 template <typename E>
 __device__ __noinline__ uint32_t verify_dense(const E *__restrict__ plane, int64_t nb, int zmax, int K, bool anchored, int H,
                                               int row, int64_t r0, int64_t rmax, uint32_t cells) {
@@ -463,8 +461,9 @@ __device__ __noinline__ uint32_t verify_dense(const E *__restrict__ plane, int64
 // gathers in flight together: one or two round trips to L2 per three cells.  (One lane per cell, its
 // neighbours one after another, cost up to 8 H dependent round trips for each cell of a lane, and the
 // cells along a strong signal were often all in one lane.)  From DENSE_CELLS cells on the
-// gathers' sectors cost more than their latency: verify_dense (FP32, N = 2^23, 11 million peaks, mostly
-// units of 30 to 200 cells: 12 ms with the line at 32, 6.6 at 128, 6.0 at 256; in place 12.4).
+// gathers' sectors cost more than their latency: verify_dense (FP32, N = 2^23, whole call, 11 million peaks, mostly
+// units of 30 to 200 cells: 6.1 ms with the line at 32, 4.8 at 128, 4.6 at 256; 54 million: 10.7, and 28.5 without
+// verify_dense).
 constexpr int DENSE_CELLS = 256;
 template <typename E>
 __device__ __forceinline__ void verify_unit(const E *__restrict__ plane, int64_t nb, int zmax, int K, bool anchored,
@@ -519,14 +518,27 @@ __device__ __forceinline__ void verify_unit(const E *__restrict__ plane, int64_t
     if (lane < WORDS) unit_mask[u * WORDS + lane] = word;
 }
 
+// max(a, b, c), NaN when any of them is (a cell beside a NaN is no peak); three-input max.f32: sm_100 and later.
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+    float d;
+    asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 // The peaks of one level-1 unit u of row i, bins r0 .. r0 + 511, that holds a value above the threshold.  At
-// level 1 a neighbour's sum is a plane value, so a lane reads its 16 bins of the three rows as vectors (one
-// round trip for the whole unit, however many cells are above) and the bins beside them come by shuffles.
-// Out of line, the own row read again, so that the stream over the plane keeps its registers.
-// FP32, N = 2^23, 85 templates, 54 million peaks at all levels: 18.8 -> 11.0 ms with this in place of nine
-// lanes to a cell (below 256 cells a unit) or a lane to a bin.
+// level 1 a neighbour's sum is a plane value.  Two forms, both out of line and reading the own row again, so that
+// the callers' streams keep their registers:
+//  * level1_many: a lane reads its 16 bins of the three rows as vectors (one round trip for the whole unit,
+//    however many cells are above) and the bins beside them come by shuffles.  FP32, N = 2^23, 85 templates, 54
+//    million peaks at all levels: 18.8 -> 10.7 ms with this in place of nine lanes to a cell (below 256 cells a
+//    unit) or a lane to a bin.
+//  * level1_few, after a marking plane kernel: only the words of 32 bins with cells, at most LEVEL1_FEW, a lane to
+//    a bin, in a short loop.  A search with a few strong cells waits longer for level1_many's unrolled code than for
+//    its loads (N = 2^18, BF16, 4 pulse trains: k4_level1_marked 15.0 -> 9.4 us with cold caches, the search
+//    62.8 -> 60.7).
+constexpr int LEVEL1_FEW = 4;
 template <typename E>
-__device__ __noinline__ void level1_unit(const E *__restrict__ plane, int64_t nb, int K, const LevelDesc &d, int i, int64_t r0,
+__device__ __noinline__ void level1_many(const E *__restrict__ plane, int64_t nb, int K, const LevelDesc &d, int i, int64_t r0,
                                          int u, int32_t *__restrict__ unit_count, uint32_t *__restrict__ unit_mask) {
     const int lane = threadIdx.x & 31;
     const int64_t rl = r0 + LB * lane;
@@ -560,8 +572,8 @@ __device__ __noinline__ void level1_unit(const E *__restrict__ plane, int64_t nb
 #pragma unroll
         for (int e = 0; e < LB; e++) {
             const float b = e == 0 ? before : w[e == 0 ? 0 : e - 1], c = e == LB - 1 ? after : w[e == LB - 1 ? e : e + 1];
-            const bool ok = (a <= 0 ? v[e] > b : v[e] >= b) && (a < 0 ? v[e] > w[e] : v[e] >= w[e]) && (a < 0 ? v[e] > c : v[e] >= c);
-            if (!ok) pk &= ~(1u << e);
+            if (k == 0 ? !(v[e] > b && v[e] >= c) : k == 1 ? !(v[e] > max3_nan(b, w[e], c)) : !(v[e] >= max3_nan(b, w[e], c)))
+                pk &= ~(1u << e);
         }
     }
     int cnt = __popc(pk);
@@ -570,6 +582,58 @@ __device__ __noinline__ void level1_unit(const E *__restrict__ plane, int64_t nb
     const uint32_t hi = __shfl_down_sync(0xffffffffu, pk, 1);
     if (lane == 0) count_unit(unit_count, u, cnt);
     if (cnt > 0 && !(lane & 1)) unit_mask[(int64_t)u * WORDS + (lane >> 1)] = pk | (hi << 16);
+}
+
+template <typename E>
+__device__ __noinline__ bool level1_few(const E *__restrict__ plane, int64_t nb, int K, const LevelDesc &d, int i, int64_t r0,
+                                        int u, int32_t *__restrict__ unit_count, uint32_t *__restrict__ unit_mask) {
+    const int lane = threadIdx.x & 31;
+    uint32_t above = 0;                                  // the lane's 16 bins
+    {
+        typename Fmt<E>::Raw raw;
+        Fmt<E>::load_raw(plane + (int64_t)i * nb + r0 + LB * lane, raw);
+        float v[LB];
+        Fmt<E>::widen(raw, v);
+#pragma unroll
+        for (int e = 0; e < LB; e++)
+            if (v[e] > d.thr) above |= 1u << e;
+    }
+    // word w of the unit in lane w < 16
+    const uint32_t cells = __shfl_sync(0xffffffffu, above, (2 * lane) & 31) | __shfl_sync(0xffffffffu, above, (2 * lane + 1) & 31) << 16;
+    uint32_t live = __ballot_sync(0xffffffffu, lane < WORDS && cells != 0);
+    if (__popc(live) > LEVEL1_FEW) return false;
+    uint32_t word = 0;
+#pragma unroll 1
+    for (; live; live &= live - 1) {
+        const int w = __ffs(live) - 1;
+        const int64_t r = r0 + 32 * w + lane;
+        const E *p = plane + (int64_t)i * nb + r;
+        const int side = lane == 0 ? -1 : 1;             // lanes 0 and 31 read the bin beside the word, too
+        const bool edge = (lane == 0 && r > 0) || (lane == 31 && r < d.rmax);
+        float v[3], o[3];                                // rows i - 1, i, i + 1; an undefined neighbour loses
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            const bool row = i + a > 0 && i + a <= K;
+            v[a] = row ? ld_plane(p, (a - 1) * nb) : -INFINITY;
+            o[a] = row && edge ? ld_plane(p, (a - 1) * nb + side) : -INFINITY;
+        }
+        bool ok = (__shfl_sync(0xffffffffu, cells, w) >> lane) & 1u;
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            float b = __shfl_up_sync(0xffffffffu, v[a], 1), c = __shfl_down_sync(0xffffffffu, v[a], 1);
+            if (lane == 0) b = o[a];
+            if (lane == 31) c = o[a];
+            if (a == 0) ok = ok && v[1] > b && v[1] > v[0] && v[1] > c;
+            if (a == 1) ok = ok && v[1] > b && v[1] >= c;
+            if (a == 2) ok = ok && v[1] >= b && v[1] >= v[2] && v[1] >= c;
+        }
+        const uint32_t m = __ballot_sync(0xffffffffu, ok);
+        if (lane == w) word = m;
+    }
+    const int cnt = (int)__reduce_add_sync(0xffffffffu, __popc(word));
+    if (lane == 0) count_unit(unit_count, u, cnt);
+    if (cnt > 0 && lane < WORDS) unit_mask[(int64_t)u * WORDS + lane] = word;
+    return true;
 }
 
 // Level 1 over the whole plane: a pure stream.  Grid (ceil(chunks1 / (DETECT_WARPS * CPW1)), K);
@@ -601,7 +665,7 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_L1_MIN_BLOCKS) k4_l
     }
     for (; hot; hot &= hot - 1) {
         const int c = c0 + __ffs(hot) - 1;
-        level1_unit<E>(plane, nb, K, d, i, (int64_t)c * CB, (int)d.unit0 + i * (int)d.chunks + c, unit_count, unit_mask);
+        level1_many<E>(plane, nb, K, d, i, (int64_t)c * CB, (int)d.unit0 + i * (int)d.chunks + c, unit_count, unit_mask);
     }
 }
 
@@ -716,14 +780,16 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32) k4_level1_marked(const E *_
     while (todo) {
         const int64_t uu = u0 + (__ffs(todo) - 1);
         todo &= todo - 1;
-        const int i = (int)(uu / d.chunks);
+        const int i = (int)(uu / d.chunks), unit = (int)(d.unit0 + uu);
         const int64_t r0 = (uu - (int64_t)i * d.chunks) * CB;
         typename Fmt<E>::Raw raw;                    // most are marked for level 2's sake (mark_threshold)
         Fmt<E>::load_raw(plane + (int64_t)i * nb + r0 + LB * lane, raw);
-        if (__any_sync(0xffffffffu, Fmt<E>::max16(raw) > d.thr))
-            level1_unit<E>(plane, nb, K, d, i, r0, (int)(d.unit0 + uu), unit_count, unit_mask);
-        else if (lane == 0)
-            unit_count[d.unit0 + uu] = 0;
+        if (__any_sync(0xffffffffu, Fmt<E>::max16(raw) > d.thr)) {
+            if (!level1_few<E>(plane, nb, K, d, i, r0, unit, unit_count, unit_mask))
+                level1_many<E>(plane, nb, K, d, i, r0, unit, unit_count, unit_mask);
+        } else if (lane == 0) {
+            unit_count[unit] = 0;
+        }
     }
 }
 
@@ -943,8 +1009,10 @@ __global__ void __launch_bounds__(DETECT_WARPS * 32, FDAS_K4_MIN_BLOCKS) k4a_lev
 // The units left to be tested (count -1), one warp each: those on the list, or, when it did not hold all
 // units, every one in the order of the level search (order: entries row << 16 | chunk group, rows from
 // lt.lev[1].i_lo; nullptr: column by column), so that the sums around a unit's cells find their sectors in
-// L2 (FP32, N = 2^23, 42 million peaks: 37 ms in the units' order, 20 in the search's).  Four blocks to an SM at 64 registers: the
-// gathers' latency is hidden by warps (anchored sums, N = 2^21, 19 million peaks: 13.8 ms with two, 12.0).
+// L2 (FP32, N = 2^23, 42 million peaks, when level 1 was tested here too: 37 ms in the units' order, 20 in the
+// search's).  Four blocks to an SM at 64 registers, which spill some (404 bytes of stores on FP32 planes, 724 on
+// BF16): the gathers' latency is hidden by warps (anchored sums, N = 2^21, 19 million peaks: 13.0 ms with two blocks,
+// 11.4; plain sums on short planes, N = 2^18, 333943 peaks: 0.27 ms with two, 0.36).
 constexpr int VERIFY_WARPS = 8;
 template <typename E>
 __global__ void __launch_bounds__(VERIFY_WARPS * 32, 4) k4_verify(const E *__restrict__ plane, int64_t nb, int zmax, int K,
