@@ -128,6 +128,11 @@ __device__ __forceinline__ void k1_sum_and_finalize(float acc, double *red, doub
     }
 }
 
+// Lengths of pass B that a search launched early can have (launch_early_bins(): two passes of at most 512 on 152
+// SMs).  The longer ones keep their loads on the read-only path and wait for nothing: with the wait and plain
+// loads they spilled, and took 1 to 2 % longer (N = 2^25: 472 -> 480 us for the whole spectrum).
+constexpr bool k1_early_b(int M2) { return M2 <= 512; }
+
 // Groups 0 .. C2-1 take rows a = p C2 + g; groups C2 .. 2 C2 - 1 their partners M1 - a (row 0,
 // its own partner, lends its partner slot to row M1/2, the other self-partnered row).
 template <int M2>
@@ -135,8 +140,8 @@ __global__ void __launch_bounds__(2 * k1_groups_b(M2) * (M2 / 32), FDAS_K1B_MIN_
                                                                          const float2 *__restrict__ tw,
                                                                          const float2 *__restrict__ lo,
                                                                          const float2 *__restrict__ hi,
-                                                                         float2 *X,
-                                                                         double *partial, int M1,
+                                                                         float2 *__restrict__ X,
+                                                                         double *__restrict__ partial, int M1,
                                                                          unsigned int *__restrict__ ticket, int64_t nb,
                                                                          double sigma2_fixed, double *__restrict__ sigma2_out,
                                                                          float *__restrict__ scale_out, bool release) {
@@ -150,11 +155,16 @@ __global__ void __launch_bounds__(2 * k1_groups_b(M2) * (M2 / 32), FDAS_K1B_MIN_
     float2 *sm = smb + g * E;
     __shared__ float2 w64[32];            // W_N^{M1 T i} = W_64^i
     for (int i = threadIdx.x; i < 32; i += G * T) w64[i] = twN(lo, hi, (int64_t)M1 * T * i);
-    grid_wait();
-    if (release) grid_release();
+    if constexpr (k1_early_b(M2)) {
+        grid_wait();
+        if (release) grid_release();
+    }
     float2 v[32];
 #pragma unroll
-    for (int i = 0; i < 32; i++) v[i] = B[(int64_t)row * M2 + t + i * T];
+    for (int i = 0; i < 32; i++) {
+        const float2 *b = B + (int64_t)row * M2 + t + i * T;
+        v[i] = k1_early_b(M2) ? *b : __ldg(b);
+    }
     block_fft<M2>(v, sm, tw, t);
     // the last FFT stage works in registers and the previous exchange ended with a barrier
 #pragma unroll
@@ -262,7 +272,7 @@ cudaError_t run_pass_b(const Plan &p, const float2 *B, float2 *X, double *partia
     auto kern = k1_pass_b<M2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_after(early, kern, p.M1 / (2 * C2), 2 * C2 * (M2 / 32), smem, st, B, p.d_tw, p.d_twn_lo, p.d_twn_hi, X, partial, p.M1,
+    return launch_after(early && k1_early_b(M2), kern, p.M1 / (2 * C2), 2 * C2 * (M2 / 32), smem, st, B, p.d_tw, p.d_twn_lo, p.d_twn_hi, X, partial, p.M1,
                         ticket, p.nb, p.cfg.sigma2, sigma2, scale, release_at_once(p));
 }
 
