@@ -331,7 +331,9 @@ fdas_status fdas_interp_power(fdas_plan_t plan, const float *d_xhat, const fdas_
  * response), scaled to |dr| <= 1/4 and |dz| <= 1 and halved up to three times until P does not
  * decrease; a candidate stops early when no such step exists.
  *   d_out    n refined points (may equal d_in).
- *   d_power  (nullable) n x 3 doubles: FP64 P, dP/dr, dP/dz at the refined point.
+ *   d_power  (nullable) n x 3 doubles: FP64 P, dP/dr, dP/dz at the refined point.  The ascent has
+ *            its own FP64 evaluation: fdas_interp_power with fp64 = 1 at the same point agrees to
+ *            about 1e-14 of the power, not bit for bit.
  *   d_evals  (nullable) n int32: power evaluations spent on each candidate.
  * A seed that fdas_interp_power would reject is copied unchanged with NaN power.
  * Device pointers 8-byte aligned (d_evals 4).  Needs no templates.

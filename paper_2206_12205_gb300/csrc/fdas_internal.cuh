@@ -134,18 +134,18 @@ void gauss_legendre(int n, double *xs, double *ws);
 // last of those finishes; grid_wait() then holds it until that one has completed and its writes are
 // visible.  Its blocks pass grid_wait() before they touch memory that other kernels write or read, and
 // call grid_release() (which lets the next kernel's blocks in, once every block has called it or
-// exited) only after that: so when a kernel starts, all but the last kernel before it have completed,
+// exited) only after that, or are launched plainly (k1_pass_a, k4_level1_marked): so when a kernel starts, all but the last kernel before it have completed,
 // and only what that last one writes has to be read with plain loads instead of the read-only path.
 //   early: a search by itself of at most launch_early_bins() bins, whose kernels are short enough that
-// the gaps between them count (N = 2^16, FP32, 64 taps: 50.5 -> 35 us; N = 2^18, BF16: 72 -> 62 us; BF16
-// N = 2^19: 82 -> 75 us).  On larger ones a plane kernel that waits beside the segment FFTs' last waves
+// the gaps between them count (N = 2^16, FP32, 64 taps: 50.5 -> 35 us; N = 2^18, BF16: 72 -> 61 us; BF16
+// N = 2^19: 81 -> 68 us).  On larger ones a plane kernel that waits beside the segment FFTs' last waves
 // costs more than the gap (BF16, N = 2^20: 116 -> 123 us; N = 2^23: 588 -> 608 us), and in batches blocks that wait keep the
 // other lanes' out (12 series of 2^21, 3 lanes: 3.32 -> 3.52 ms); these launch plainly, which makes
 // both calls no-ops.
 //   early_tail: the peak search's list and output kernels (k4_compact, k4_verify, k4_emit_listed) in a call
 // by itself, of any size.  They wait for little, and what they save is the gap: k4_verify and k4_compact,
 // launched plainly, had made calls with few peaks slower than one kernel that did it all (fdas_peaks, FP32,
-// N = 2^16: 21.8 us once, 24.8 -> 20.1; search, FP16, N = 2^20, 21 templates: 69.9 once, 71.8 -> 66).
+// N = 2^16: 21.8 us once, 24.8 -> 20.3; search, FP16, N = 2^20, 21 templates: 71.7 once, 72.7 -> 67.6).
 inline int64_t launch_early_bins(int device) {
     int sms = 152;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device >= 0 ? device : 0);

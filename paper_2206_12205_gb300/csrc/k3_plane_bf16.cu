@@ -585,8 +585,10 @@ __global__ void __launch_bounds__(WS_THREADS, 1) k3_plane_tc(const uint4 *Y, con
 //   epilogue 2:  |D2|^2 -> FP32 plane
 // F1, F2 hi and lo take 128 KB of shared memory, so A1 and A2 have one slot each: stage 1 of item
 // k + 1 runs while epilogue 1 writes A2 of item k, stage 2 of item k while the producer writes A1 of
-// item k + 2.  The MMAs bound it: 48 of 64 cycles an item = 3072 cycles.  N = 2^21, 85 templates,
-// 256 taps: 0.849 -> 0.25 ms (before: one item at a time and a CTA-wide barrier between the steps).
+// item k + 2.  The MMAs are its floor: 48 of 64 cycles an item = 3072 cycles.  An item takes
+// 6050 (ncu, N = 2^21, 85 templates, 256 taps: tensor pipe 55 % active, shared-memory data path 55 %, issue 54 %):
+// with one slot of A2, epilogue 1's stores of an item and stage 2 of the item before it take turns.
+// There: 0.849 -> 0.243 ms (before: one item at a time and a CTA-wide barrier between the steps).
 __device__ __forceinline__ void split_bf16x2(float re, float im, uint32_t &hi, uint32_t &lo) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(re, im);
     const float2 hf = __bfloat1622float2(h);
@@ -596,7 +598,8 @@ __device__ __forceinline__ void split_bf16x2(float re, float im, uint32_t &hi, u
 }
 
 // Registers at launch 72 a thread; 128 x 56 + 256 x 88 + 256 x 72 + 256 x 64 = 896 x 72 (the
-// producers hold the FP32 loads of the next eight points while they split the current ones).
+// producers hold the FP32 loads of the next eight points while they split the current ones; 72 is short of
+// what the compiler would take, and it spills 52 bytes).
 constexpr int SP_REG_MMA = 56, SP_REG_PROD = 88, SP_REG_E1 = 72, SP_REG_E2 = 64;
 static_assert(128 * SP_REG_MMA + 256 * (SP_REG_PROD + SP_REG_E1 + SP_REG_E2) == WS_THREADS * REG_LAUNCH,
               "register split must add up to the launch allocation");

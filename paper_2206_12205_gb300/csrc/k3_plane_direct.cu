@@ -25,10 +25,12 @@
 // writes 256 consecutive bytes where one 2-byte store per set touched every sector four times.
 // Two accumulator slots in TMEM, two window slots in shared memory, every mbarrier wait bounded
 // (timeout -> FDAS_DEV_TIMEOUT, MMAs drained, TMEM freed).
-// The MMAs are its floor: each reads 4 KB of window and 16 N bytes of taps from shared memory (the
-// operand rate is 128 bytes a cycle), 4 m / 8 of them a tile.  N = 2^22, 21 templates, 64 taps: 95 us
-// and a separate packing pass of 8 us -> 55 us (before: one window warp on dependent 4-byte loads,
-// 2-byte stores 8 bytes apart).
+// The MMAs' operand reads are its floor: each takes 4 KB of window and 16 N bytes of taps from shared memory (128
+// bytes a cycle), 4 m / 8 of them a tile.  N = 2^22, 21 templates, 64 taps: 95 us and a separate packing pass of 8 us
+// -> 56 us (before: one window warp on dependent 4-byte loads, 2-byte stores 8 bytes apart).  That is 4100 cycles a
+// tile against 1220 of operand reads, and no unit is full (ncu: tensor pipe 20 %, issue 39 %, shared-memory data path
+// 12 %, DRAM 10 %): what paces it is the hand-over between the roles, which has not been timed role by role.
+// With 85 templates and 256 taps the MMAs come closer to filling it: 70 % of the burst BF16 rate (N = 2^23: 0.546 ms).
 #include <cuda_fp8.h>
 
 #include "fdas_internal.cuh"

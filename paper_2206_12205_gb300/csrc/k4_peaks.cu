@@ -1145,7 +1145,8 @@ __device__ __forceinline__ int32_t block_excl_scan(int32_t c, int32_t *warp_tot,
 // offset; a few MB read from L2 per block, no communication between blocks), then scans its
 // range, 4096 units a round at most, and deals the round's non-empty units to its warps.  Shares of
 // whole rounds left a plane of 10^4 units to two or three blocks (level 1 alone, FP32, N = 2^18, 27296 peaks:
-// 395 -> 55 us for the call; N = 2^16, 312797 peaks: 886 -> 35 us).  The last block (or block 0
+// 395 -> 55 us for the call; N = 2^16, 312797 peaks: 886 -> 35 us).  1024 threads leave 64 registers: emit_unit's
+// 16 gathers in flight spill some 130 bytes.  The last block (or block 0
 // on the listed path) writes the total and the overflow flag.
 static_assert(PEAK_LIST_CAP == 4 * 1024, "a round of the scan: four units a thread");
 template <typename E>

@@ -48,8 +48,11 @@
 //  * conversions and branch decisions in FP32 and integer arithmetic;
 //  * the scalar work (square roots, divisions, the phase at u = 1) lane-parallel: a warp takes a group
 //    of points, one per lane, then evaluates them one after another with all lanes on the taps.
-// About 65 FP64 instructions per tap and lane where the form above takes 600.  4096 points, 256 taps,
-// |z| <= 84: 1000 -> 270 us, and closer to the exact sums (relative error 3e-15 against 1e-14).
+// About 65 FP64 instructions per near tap and lane where the form above takes 600.  4096 points, 256 taps,
+// |z| <= 84: 1000 -> 270 us, and closer to the exact sums (relative error 3e-15 against 1e-14).  There a step of 32
+// taps executes 118 (a warp with near and far taps runs both, and the points' scalar work is in it), and the FP64
+// pipe is 87 % busy on an SM that has a block, 69 % over the kernel: 256 blocks at two to an SM leave 48 of 152 SMs
+// with one.
 // k5_refine keeps the first form for its FP64 step: on a converged candidate whether that step is
 // taken hangs on the last bits of P, so another evaluation changes evaluation counts and, along the
 // degenerate direction, points.

@@ -50,7 +50,9 @@ def interp_power(plan, xhat, r: torch.Tensor, z: torch.Tensor, fp64: bool = Fals
 def refine(plan, xhat, seeds: torch.Tensor, steps: int = 20):
     """Refine (n, 2) float64 seeds (r, z) on the device.
 
-    Returns (points (n, 2), power (n, 3): FP64 P, dP/dr, dP/dz at each point, evals (n,))."""
+    Returns (points (n, 2), power (n, 3): FP64 P, dP/dr, dP/dz at each point, evals (n,)).  The power
+    agrees with interp_power(fp64=True) at the point to about 1e-14, not bit for bit (the ascent has
+    its own evaluation)."""
     n = int(seeds.shape[0])
     dev = seeds.device
     out = torch.empty(n, 2, dtype=torch.float64, device=dev)
